@@ -60,6 +60,14 @@ constexpr float KMEM = 16.f * KU;
 constexpr float KH = 1.953125e-03f;         // 2^-9
 constexpr float EH = 9.5367431640625e-07f;  // 2^-20
 constexpr float MAGH = 16384.f;
+// Half-precision reach rows.  The screened kernel takes the other reach rows
+// of a pair in FP16 by the same bound, in both directions, with KHF = 17/16
+// times the 2^-10 of the bound (the single roundings of the band's own FP32
+// arithmetic are far below the sixteenth): a maximum above
+// 1 + (KR + KHF) * magnitude + EH certainly fails, one below 1 minus that
+// certainly passes.  What the band does not decide (about 1% of the screened
+// checks) is evaluated in FP32.
+constexpr float KHF = 1.03759765625e-03f;  // 17/16 * 2^-10
 // FP32 cost conditioning.  A cost is a sum of segment norms of (start half +
 // end half) rows; its rounding error stays below about 1.2 u times the sum of
 // |half| over all rows (measured over every feasible check of the 2-D and 3-D
@@ -125,6 +133,23 @@ struct Shape {
     static constexpr int RAX = (G >= 1 ? PD : 0) + (G >= 2 ? PD - 1 : 0) + (G >= 3 ? PD - 2 : 0) + (G >= 4 ? PD - 3 : 0);
     static constexpr int NI = PD - 1;
     static constexpr int TG = 2 * G;
+    // The FP32 table's row order: derivative k = G first, per derivative the
+    // interior control points j = 1 .. PD-k-1, then j = 0, then j = PD-k.
+    static constexpr int order_of(int r) {  // k of table row r
+        int k = G;
+        while (r >= PD - k + 1) r -= PD - k-- + 1;
+        return k;
+    }
+    static constexpr int point_of(int r) {  // j of table row r
+        int k = G;
+        while (r >= PD - k + 1) r -= PD - k-- + 1;
+        return r == PD - k ? PD - k : (r == PD - k - 1 ? 0 : r + 1);
+    }
+    static constexpr int table_row(int k, int j) {
+        for (int r = 0; r < RAX; ++r)
+            if (order_of(r) == k && point_of(r) == j) return r;
+        return -1;
+    }
 };
 
 // Member-list entries carry the state id in bits 0..30 and, in bit 31, whether
@@ -832,17 +857,30 @@ DEVI void pair_phase(const BuildParams& P, const Item& itd, int t, int T, int gi
 template <int G, int PD>
 struct Screen {
     static constexpr int NS = 3;
-    // reach-row index (k-major canonical layout): k = 2, j = G-2 and j = PD-G; k = 1, j = (PD-1)/2
-    static constexpr int row(int s) { return s == 0 ? PD + (G - 2) : (s == 1 ? PD + (PD - G) : (PD - 1) / 2); }
-    static constexpr int index(int rr) { return rr == row(0) ? 0 : (rr == row(1) ? 1 : (rr == row(2) ? 2 : -1)); }
+    // table rows of k = 2, j = G-2 and j = PD-G; k = 1, j = (PD-1)/2
+    static constexpr int row(int s) {
+        return s == 0 ? Shape<G, PD>::table_row(2, G - 2)
+                      : (s == 1 ? Shape<G, PD>::table_row(2, PD - G) : Shape<G, PD>::table_row(1, (PD - 1) / 2));
+    }
+    // 2 bits a table row: 1 + its place in the screen, 0 for the other rows
+    // (a constant, so that the unrolled loops fold it)
+    static constexpr unsigned long long places() {
+        unsigned long long v = 0;
+        for (int i = 0; i < NS; ++i) v |= (unsigned long long)(i + 1) << (2 * row(i));
+        return v;
+    }
+    static constexpr unsigned long long PLACES = places();
+    static constexpr int index(int rr) { return (int)((PLACES >> (2 * rr)) & 3) - 1; }
 };
 
 // The screen of one 4x4 micro-tile on the screen row-axes in FP16, stored
 // [row][state]: start states as (h, h) pairs, end states as single halves, so
 // one packed add gives two pairs' sums.  Returns the live pairs that do not
-// certainly fail there (the band of the FP32 sum widened by the FP16 error).
+// certainly fail there (the band of the FP32 sum widened by the FP16 error);
+// the FP16 values are sc times the rows.
 template <int M, int G, int PD>
-DEVI uint32_t screen_tile(int T, int gi, int gj, uint32_t live, const __half2* SCL, const __half* SCR, const float* magR) {
+DEVI uint32_t screen_tile(int T, int gi, int gj, uint32_t live, float sc, const __half2* SCL, const __half* SCR,
+                          const float* magR) {
     __half2 rm[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) rm[q] = __float2half2_rn(0.f);
@@ -870,8 +908,8 @@ DEVI uint32_t screen_tile(int T, int gi, int gj, uint32_t live, const __half2* S
             const int q = qa * 4 + qb;
             const __half2 m2 = rm[qa * 2 + (qb >> 1)];
             const float r = (qb & 1) ? __high2float(m2) : __low2float(m2);
-            const float ms = magR[4 * gi + qa] + magR[T + 4 * gj + qb];
-            if (!(r <= 1.f + (KR + KH) * ms + EH) && ms <= MAGH) fail |= 1u << q;
+            const float ms = sc * (magR[4 * gi + qa] + magR[T + 4 * gj + qb]);
+            if (!(r <= sc + (KR + KH) * ms + EH) && ms <= MAGH) fail |= 1u << q;
         }
     return live & ~fail;
 }
@@ -1141,73 +1179,194 @@ __global__ void __launch_bounds__(256, 2) k_pairs_fast(BuildParams P) {
 // ---------------------------------------------------------------------------
 // Screened FP32 pair kernel (the default one).  Same persistent item loop as
 // the one-group kernel, in four phases per duration:
-//   1. reach halves, stored per state ([state][row], rows padded to 16-byte
-//      quads, per-state stride = 4 mod 8 floats so that quad loads of
-//      different states fall in different bank groups); the screen row-axes
-//      also in FP16, stored [row][state] for the micro-tile screen; the
-//      interior control points' halves; the cost rows' magnitudes;
+//   1. per state an FP16 record ([state][word], whole 16-byte quads, stride
+//      = 4 mod 8 words so that quad loads of different states fall in
+//      different bank groups) of the reach row-axes that depend on both
+//      boundary states, the interior control points' halves in FP32 beside
+//      it; the rows that one state fixes alone reduced to their maximum; the
+//      screen row-axes also stored [row][state] for the micro-tile screen;
 //   2. screen of every 4x4 micro-tile; pairs that do not certainly fail are
 //      appended to list 1 (shared memory);
-//   3. every reach row of the list-1 pairs (four per 16-byte load) and, for
-//      those that pass, every polytope row at every interior control point,
-//      one pair per thread; feasible pairs go to list 2, ambiguous ones to
-//      the FP64 re-check;
-//   4. costs of the list-2 pairs from their two staged states and the atomic
-//      merge into the pair slots.
-// Maxima are order-free and the reach sums and costs keep the reference
-// order, so slots and costs equal those of the other FP32 kernels; the free
-// margins take fewer roundings within the same band, so only the set of
-// ambiguous margins re-checked in FP64 can differ.
+//   3. the list-1 pairs, one per thread: every reach row in packed FP16 from
+//      two records, with a band that decides all but about 1% of them (those
+//      go through every row in FP32, a warp to a pair), and, for pairs that
+//      pass, every polytope row at every interior control point in FP32.
+//      Feasible pairs go to list 2, ambiguous ones to the FP64 re-check.
+//   4. costs of the list-2 pairs, from cost halves staged in place of the
+//      records or, when the list is short, from the two staged states, and
+//      the atomic merge into the pair slots.
+// Decisions are those of the FP32 rows: FP16 and the box rows only settle what
+// they settle for certain.  Maxima are order-free and the costs keep the
+// reference order, so slots and costs equal those of the other FP32 kernels;
+// the free margins take fewer roundings within the same band, so only the set
+// of ambiguous margins re-checked in FP64 can differ.
+//
+// Bound by issue and by the spread of the work between its barriers (24 warps
+// an SM at 80 registers; a fourth CTA at 64 registers gained nothing).  On the
+// 3-D workload (8192 states, 64 polytopes, 16 durations, 29.2 M checks) 266 ->
+// 208 us and 211 -> 144 M warp instructions against FP32 rows read from both
+// states for every screened pair: FP16 rows halve that traffic, the rows that
+// one state fixes leave the pair loop (a third of them), rows along an axis
+// take the extreme coordinate (a fifth of the work of a general row), costs
+// from staged halves take 270 instead of 750 instructions a pair, and the
+// screen's three rows are the ones that reject most (it passes 1.4% more pairs
+// than the whole reach test; 24% more with the rows first chosen).  Phases by
+// leaving them out: set-up 35, halves 27, screen 26, rows 75, costs 45 us.
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int pad_odd4(int n) { return ((n + 3) / 8) * 8 + 4; }  // >= n, = 4 mod 8
 
-// per-state stride of the interior control points' halves
-__host__ __device__ inline int sc_free_stride(int NI, int M) {
-    return pad_odd4((NI * M + 3) & ~3);  // the interior control points' halves
-}
-
 template <int M, int G, int PD>
 struct ScShape {
-    using S = Shape<G, PD>;
-    static constexpr int RR = M * S::RAX;        // reach row-axes
-    static constexpr int RQ = (RR + 3) / 4;      // their 16-byte quads
-    static constexpr int RH = (RQ + 1) / 2;      // quads of the first half-unit
-    static constexpr int SU = pad_odd4(4 * RQ);  // per-state stride of the reach halves
+    // The reach row of derivative k, control point j depends on the start
+    // state alone when j + k <= G-1 (side 0), on the end state alone when
+    // j >= PD-G+1 (side 1), else on both: the first and last G control points
+    // are fixed by one boundary state, for either interior reading.
+    static constexpr int side(int r) {
+        const int k = Shape<G, PD>::order_of(r), j = Shape<G, PD>::point_of(r);
+        return j + k <= G - 1 ? 0 : (j >= PD - G + 1 ? 1 : 2);
+    }
+    static constexpr int count(int sd) {
+        int n = 0;
+        for (int r = 0; r < Shape<G, PD>::RAX; ++r) n += side(r) == sd ? 1 : 0;
+        return n;
+    }
+    // the rows of a side, 5 bits each (constants, so that the unrolled loops fold them)
+    static constexpr unsigned long long rows(int sd) {
+        unsigned long long v = 0;
+        int n = 0;
+        for (int r = 0; r < Shape<G, PD>::RAX; ++r)
+            if (side(r) == sd) v |= (unsigned long long)r << (5 * n++);
+        return v;
+    }
+    static constexpr unsigned long long ROWS0 = rows(0), ROWS1 = rows(1), ROWS2 = rows(2);
+    static constexpr int row(int sd, int i) { return (int)(((sd == 0 ? ROWS0 : (sd == 1 ? ROWS1 : ROWS2)) >> (5 * i)) & 31); }
+    static_assert(count(2) <= 12 && Shape<G, PD>::RAX <= 32, "5 bits a row in 64");
+    static constexpr int NB = count(2);             // rows of both states
+    static constexpr int N1 = count(0);             // rows of one state (as many for either side)
+    static constexpr int RW = (NB * M + 1) / 2;     // their row-axes, two FP16 values a word
+    static constexpr int RQ = (RW + 3) / 4;         // 16-byte quads of a record
+    static constexpr int NP = (Shape<G, PD>::NI * M + 3) & ~3;  // floats of the interior control points' halves
+    static constexpr int QH0 = (2 * RW + (Shape<G, PD>::NI + N1) * M + 8) / 16;  // quads of the first half-unit: half the rows
+    static constexpr int QH = QH0 < 1 ? 1 : (QH0 > RQ ? RQ : QH0);
+    static constexpr int SU = pad_odd4(4 * RQ);     // per-state stride of the records (words)
+    static constexpr int SF = pad_odd4(NP);         // per-state stride of the points' halves
     static constexpr int NS = Screen<G, PD>::NS * M;
-    static constexpr int XS = pad_odd4(M * G);   // per-state stride of the staged states
+    static constexpr int XS = pad_odd4(M * G);      // per-state stride of the staged states
+    static_assert(count(0) == count(1), "the rows mirror");
 };
 
-// Reach halves of one state for quads [Q0, Q1): row-axis q = rr*M + a holds
-// sum_c H[rr][side][c] x[c][a]; rows past RR are 0 (neutral in max |u + w|).
-// The screen row-axes also go, rounded to FP16, to the screen arrays dS.
+// One half (start or end, by the table pointer) of a row-axis:
+// sum_c h[c] x[c][a] with FMA, left to right.
+template <int M, int G>
+DEVI float row_half(const float* h4, const float* x, int a) {
+    const float4 h = *reinterpret_cast<const float4*>(h4);
+    float v = h.x * x[a];
+    if (G > 1) v = fmaf(h.y, x[M + a], v);
+    if (G > 2) v = fmaf(h.z, x[2 * M + a], v);
+    if (G > 3) v = fmaf(h.w, x[3 * M + a], v);
+    return v;
+}
+
+DEVI unsigned pack_h2(float lo, float hi) {
+    const __half2 h = __floats2half2_rn(lo, hi);
+    unsigned u;
+    __builtin_memcpy(&u, &h, 4);
+    return u;
+}
+DEVI __half2 as_h2(unsigned u) {
+    __half2 h;
+    __builtin_memcpy(&h, &u, 4);
+    return h;
+}
+
+// Quads [Q0, Q1) of one state's FP16 record: the row-axes of both states, two
+// a word (value 2w in the low half; 0 past the end, neutral in max |u + w|).
+// The screen row-axes also go to the screen arrays, (h, h) for start states,
+// h for end states.
 template <int M, int G, int PD, int Q0, int Q1>
-DEVI void reach_quads(const float (&x)[M * G], const float* trow, float* dU, void* dS, int ls, bool right, int T) {
-    constexpr int RR = ScShape<M, G, PD>::RR;
+DEVI void record_quads(const float (&x)[M * G], const float* tab, unsigned* dU, void* dS, int ls, bool right, int T) {
+    using SS = ScShape<M, G, PD>;
+    const float* trow = tab + (right ? 4 : 0);
 #pragma unroll
     for (int qd = Q0; qd < Q1; ++qd) {
-        float w[4];
+        unsigned w4[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int q = 4 * qd + j;
-            w[j] = 0.f;
-            if (q < RR) {
-                const int rr = q / M, a = q % M;
-                const float4 h = *reinterpret_cast<const float4*>(trow + rr * 8);
-                float v = h.x * x[a];
-                if (G > 1) v = fmaf(h.y, x[M + a], v);
-                if (G > 2) v = fmaf(h.z, x[2 * M + a], v);
-                if (G > 3) v = fmaf(h.w, x[3 * M + a], v);
-                w[j] = v;
-                const int si = Screen<G, PD>::index(rr);
-                if (si >= 0) {  // screen row-axis in FP16: (h, h) for start states, h for end states
-                    const __half hv = __float2half_rn(v);
-                    if (right) reinterpret_cast<__half*>(dS)[(si * M + a) * T + ls] = hv;
-                    else reinterpret_cast<__half2*>(dS)[(si * M + a) * T + ls] = __halves2half2(hv, hv);
+            const int w = 4 * qd + j;
+            float v[2] = {0.f, 0.f};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (w < SS::RW) {
+                    const int q = 2 * w + h;
+                    if (q < SS::NB * M) {
+                        const int rr = SS::row(2, q / M), a = q % M;
+                        v[h] = row_half<M, G>(trow + rr * 8, x, a);
+                        const int si = Screen<G, PD>::index(rr);
+                        if (si >= 0) {
+                            const __half hv = __float2half_rn(v[h]);
+                            if (right) reinterpret_cast<__half*>(dS)[(si * M + a) * T + ls] = hv;
+                            else reinterpret_cast<__half2*>(dS)[(si * M + a) * T + ls] = __halves2half2(hv, hv);
+                        }
+                    }
                 }
             }
+            w4[j] = pack_h2(v[0], v[1]);
         }
-        *reinterpret_cast<float4*>(dU + 4 * qd) = make_float4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dU + 4 * qd) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
     }
+}
+
+// Largest |row| over the rows that this state alone fixes (FP32; the other
+// half of such a row is exactly 0).
+template <int M, int G, int PD>
+DEVI float single_max(const float (&x)[M * G], const float* tab, bool right) {
+    using SS = ScShape<M, G, PD>;
+    float mx = 0.f;
+#pragma unroll
+    for (int i = 0; i < SS::N1; ++i) {
+        const int rr = right ? SS::row(1, i) : SS::row(0, i);
+#pragma unroll
+        for (int a = 0; a < M; ++a) mx = fmaxf(mx, fabsf(row_half<M, G>(tab + rr * 8 + (right ? 4 : 0), x, a)));
+    }
+    return mx;
+}
+
+// Largest |reach row| of one pair in FP32, by a whole warp (lanes over the rows).
+template <int M, int G, int PD>
+DEVI float pair_reach_f32(const float* xi, const float* xj, const float* tab, int lane) {
+    float rm = 0.f;
+    for (int u = lane; u < Shape<G, PD>::RAX * M; u += 32) {
+        const float* h = tab + (u / M) * 8;
+        rm = fmaxf(rm, fabsf(row_half<M, G>(h, xi, u % M) + row_half<M, G>(h + 4, xj, u % M)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rm = fmaxf(rm, __shfl_xor_sync(0xffffffffu, rm, o));
+    return rm;
+}
+
+// The same by one lane.
+template <int M, int G, int PD>
+DEVI float lane_reach_f32(const float* xi, const float* xj, const float* tab) {
+    float rm = 0.f;
+#pragma unroll 1
+    for (int rr = 0; rr < Shape<G, PD>::RAX; ++rr)
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+            rm = fmaxf(rm, fabsf(row_half<M, G>(tab + rr * 8, xi, a) + row_half<M, G>(tab + rr * 8 + 4, xj, a)));
+    return rm;
+}
+
+// Interior control-point halves of one state: point l's coordinate a at
+// dP[l * M + a], zeros up to the next 16-byte quad.
+template <int M, int G, int PD>
+DEVI void point_halves(const float (&x)[M * G], const float* tab, bool right, float* dP) {
+    constexpr int NI = Shape<G, PD>::NI, NP = ScShape<M, G, PD>::NP;
+    float v[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+        v[q] = q < NI * M ? row_half<M, G>(tab + (PadTab<G, PD>::ROW_D + q / M) * 8 + (right ? 4 : 0), x, q % M) : 0.f;
+#pragma unroll
+    for (int q = 0; q < NP; q += 4) *reinterpret_cast<float4*>(dP + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
 }
 
 template <int M, int G, int PD>
@@ -1226,63 +1385,44 @@ DEVI void load_state(float (&x)[M * G], const float* xr) {
     for (int e = 0; e < M * G; ++e) x[e] = v[e];
 }
 
-// Interior control-point halves of one state for points [L0, L1): point l's
-// coordinate a, sum_c D[l][side][c] x[c][a], at dP[l * M + a]; the unit that
-// ends at NI also zeroes the padding up to the next 16-byte quad.
-template <int M, int G, int PD, int L0, int L1>
-DEVI void point_halves(const float (&x)[M * G], const float* tab, bool right, float* dP) {
-    constexpr int NI = Shape<G, PD>::NI, NP = (NI * M + 3) & ~3;
-#pragma unroll
-    for (int l = L0; l < L1; ++l) {
-        const float4 dd = *reinterpret_cast<const float4*>(tab + (PadTab<G, PD>::ROW_D + l) * 8 + (right ? 4 : 0));
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            float w = dd.x * x[a];
-            if (G > 1) w = fmaf(dd.y, x[M + a], w);
-            if (G > 2) w = fmaf(dd.z, x[2 * M + a], w);
-            if (G > 3) w = fmaf(dd.w, x[3 * M + a], w);
-            dP[l * M + a] = w;
-        }
-    }
-    if (L1 == NI) {
-#pragma unroll
-        for (int e = NI * M; e < NP; ++e) dP[e] = 0.f;
-    }
+// The FP32 cost rows of one state's side, packed: row e = d*M + a (d < DR) of
+// segment l is float l * DR * M + e, sum_c C[d][l][side][c] x[c][a].  The
+// cost conditioning sums their magnitudes in two parts, floats [0, FS) and
+// the rest: the split is at the segment boundary (PD + 1) / 2 rounded down to
+// a quad.
+template <int M, int PD, int DR>
+struct CostRows {
+    static constexpr int NF = PD * DR * M, NP = (NF + 3) & ~3;
+    static constexpr int FS0 = (((PD + 1) / 2) * DR * M) & ~3;
+    static constexpr int FS = FS0 > 0 ? FS0 : (NP > 4 ? 4 : NP);
+    static constexpr int SC = pad_odd4(NP);  // per-state stride when staged
+};
+
+template <int M, int G, int PD, int DR>
+DEVI float cost_row_half(const float* tab, const float (&x)[M * G], int f, bool right) {
+    constexpr int DRM = DR * M;
+    const int l = f / DRM, d = f % DRM / M;
+    return row_half<M, G>(tab + (PadTab<G, PD>::ROW_C + d * PD + l) * 8 + (right ? 4 : 0), x, f % M);
 }
 
-// Sum of |cost half| of one state over the floats [F0, F1) of its packed
-// cost rows (row e = d*M + a, d < DR, of segment l at float l * DR * M + e:
-// sum_c C[d][l][side][c] x[c][a]), in float order; nothing is stored.
+// Floats [F0, F1) of one state's cost halves to dC; returns the sum of their
+// magnitudes in float order.
 template <int M, int G, int PD, int DR, int F0, int F1>
-DEVI float cost_mag(const float (&x)[M * G], const float* tab, bool right) {
-    constexpr int DRM = DR * M, NF = PD * DRM;
-    static_assert(F1 > F0, "each unit takes some of the cost rows");
+DEVI float cost_halves(const float (&x)[M * G], const float* tab, bool right, float* dC) {
+    constexpr int NF = CostRows<M, PD, DR>::NF;
     float mag = 0.f;
 #pragma unroll
-    for (int f = F0; f < F1; ++f) {
-        if (f < NF) {
-            const int l = f / DRM, e = f % DRM, d = e / M, a = e % M;
-            const float4 h =
-                *reinterpret_cast<const float4*>(tab + (PadTab<G, PD>::ROW_C + d * PD + l) * 8 + (right ? 4 : 0));
-            float w = h.x * x[a];
-            if (G > 1) w = fmaf(h.y, x[M + a], w);
-            if (G > 2) w = fmaf(h.z, x[2 * M + a], w);
-            if (G > 3) w = fmaf(h.w, x[3 * M + a], w);
-            mag += fabsf(w);
+    for (int f0 = F0; f0 < F1; f0 += 4) {
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = f0 + j < NF ? cost_row_half<M, G, PD, DR>(tab, x, f0 + j, right) : 0.f;
+            mag += fabsf(v[j]);
         }
+        *reinterpret_cast<float4*>(dC + f0) = make_float4(v[0], v[1], v[2], v[3]);
     }
     return mag;
 }
-
-// The split of a state's cost rows (counted as packed floats) between its
-// two units for the magnitude sums: at the segment boundary (PD + 1) / 2
-// rounded down to a quad, the rest to the end of the padding.
-template <int M, int PD, int DR>
-struct CostSplit {
-    static constexpr int NP = (PD * DR * M + 3) & ~3;
-    static constexpr int FS0 = (((PD + 1) / 2) * DR * M) & ~3;
-    static constexpr int FS = FS0 > 0 ? FS0 : (NP > 4 ? 4 : NP);
-};
 
 // The next item for a block, or past the end once the build has failed.
 DEVI long long take_item(DevInfo* info) {
@@ -1332,11 +1472,12 @@ DEVI void stage_state_half(const void* states, bool in_f32, long long id, bool v
 
 // Control-polygon length of one pair from its two staged states: per
 // segment l the root of the sum of squares, over rows e = d*M + a (d < DR) in
-// order, of start half + end half (each sum_c C[d][l][side][c] x[c][a], the
-// table rows broadcast), summed over the PD segments in order.
+// order, of start half + end half, summed over the PD segments in order; mc:
+// the sum of all halves' magnitudes.
 template <int M, int G, int PD, int DR>
-DEVI float pair_cost_states(const float* xi, const float* xj, const float* tab) {
-    float a[M * G], b[M * G];
+DEVI float pair_cost_states(const float* xi, const float* xj, const float* tab, float& mc) {
+    constexpr int FS = CostRows<M, PD, DR>::FS;
+    float a[M * G], b[M * G], m4[4] = {0.f, 0.f, 0.f, 0.f};
     load_state<M, G, PD>(a, xi);
     load_state<M, G, PD>(b, xj);
     float cs = 0.f;
@@ -1344,57 +1485,92 @@ DEVI float pair_cost_states(const float* xi, const float* xj, const float* tab) 
     for (int l = 0; l < PD; ++l) {
         float ss = 0.f;
 #pragma unroll
-        for (int d = 0; d < DR; ++d) {
-            const float4 hl = *reinterpret_cast<const float4*>(tab + (PadTab<G, PD>::ROW_C + d * PD + l) * 8);
-            const float4 hr = *reinterpret_cast<const float4*>(tab + (PadTab<G, PD>::ROW_C + d * PD + l) * 8 + 4);
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                float cl = hl.x * a[q];
-                if (G > 1) cl = fmaf(hl.y, a[M + q], cl);
-                if (G > 2) cl = fmaf(hl.z, a[2 * M + q], cl);
-                if (G > 3) cl = fmaf(hl.w, a[3 * M + q], cl);
-                float cr = hr.x * b[q];
-                if (G > 1) cr = fmaf(hr.y, b[M + q], cr);
-                if (G > 2) cr = fmaf(hr.z, b[2 * M + q], cr);
-                if (G > 3) cr = fmaf(hr.w, b[3 * M + q], cr);
-                const float dv = cl + cr;
-                ss = fmaf(dv, dv, ss);
-            }
+        for (int f = l * DR * M; f < (l + 1) * DR * M; ++f) {
+            const float cl = cost_row_half<M, G, PD, DR>(tab, a, f, false);
+            const float cr = cost_row_half<M, G, PD, DR>(tab, b, f, true);
+            m4[f < FS ? 0 : 1] += fabsf(cl);
+            m4[f < FS ? 2 : 3] += fabsf(cr);
+            const float dv = cl + cr;
+            ss = fmaf(dv, dv, ss);
         }
         cs += sqrtf(ss);
     }
+    mc = (m4[0] + m4[1]) + (m4[2] + m4[3]);
     return cs;
 }
+
+// The same from the two states' staged halves (the same sums).
+template <int M, int PD, int DR>
+DEVI float pair_cost_halves(const float* ci, const float* cj) {
+    constexpr int NF = CostRows<M, PD, DR>::NF, DRM = DR * M;
+    float cs = 0.f, ss = 0.f;
+#pragma unroll
+    for (int f0 = 0; f0 < NF; f0 += 4) {
+        const float4 u = *reinterpret_cast<const float4*>(ci + f0);
+        const float4 w = *reinterpret_cast<const float4*>(cj + f0);
+        const float dv[4] = {u.x + w.x, u.y + w.y, u.z + w.z, u.w + w.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (f0 + j < NF) {
+                ss = fmaf(dv[j], dv[j], ss);
+                if ((f0 + j) % DRM == DRM - 1) {
+                    cs += sqrtf(ss);
+                    ss = 0.f;
+                }
+            }
+        }
+    }
+    return cs;
+}
+
+// Floats of the shared-memory region that holds the records, points, screen
+// rows and list 1, and after them the cost halves.
+template <int M, int G, int PD>
+__host__ __device__ inline int sc_front(int T, int DR) {
+    using SS = ScShape<M, G, PD>;
+    const int a = 2 * T * (SS::SU + SS::SF) + ((3 * SS::NS * T / 2 + 3) & ~3) + T * T / 2;
+    const int b = 2 * T * (DR == G ? CostRows<M, PD, G>::SC : CostRows<M, PD, 1>::SC);
+    return a > b ? a : b;
+}
+
+// Feasible pairs of a duration from which their cost halves are staged once
+// per state instead of formed per pair: staging costs a tile about 1200 warp
+// instructions and two barriers, and saves about 15 instructions a pair.
+constexpr int SC_STAGE = 160;
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
     using S = Shape<G, PD>;
     using PT = PadTab<G, PD>;
     using SS = ScShape<M, G, PD>;
-    constexpr int N_ = M * G, NI = S::NI, RQ = SS::RQ, RH = SS::RH, SU = SS::SU, NS = SS::NS, XS = SS::XS;
+    constexpr int N_ = M * G, NI = S::NI, RQ = SS::RQ, QH = SS::QH, SU = SS::SU, SF = SS::SF, NS = SS::NS, XS = SS::XS;
     static_assert(G <= 4 && M <= 3, "padded rows hold at most four coefficients");
     const int T = P.tile;  // tile side (multiple of 4, <= TILE)
     extern __shared__ __align__(16) float sm[];
     const int DR = P.cost_mode == 1 ? 1 : G;
-    const int SF = sc_free_stride(NI, M);
-    float* UL = sm;                  // [T][SU] reach halves, start states
-    float* UR = UL + T * SU;         //          end states
-    float* FL = UR + T * SU;         // [T][SF] interior control-point halves
+    unsigned* UL = reinterpret_cast<unsigned*>(sm);  // [T][SU] FP16 records, start states
+    unsigned* UR = UL + T * SU;                      //          end states
+    float* FL = reinterpret_cast<float*>(UR + T * SU);  // [T][SF] interior control-point halves
     float* FR = FL + T * SF;
-    __half2* SCL = reinterpret_cast<__half2*>(FR + T * SF);       // [NS][T] screen row-axes, start states: (h, h)
-    __half* SCR = reinterpret_cast<__half*>(FR + T * SF + NS * T);  // [NS][T] end states (half of the space used)
-    float* magR = FR + T * SF + 2 * NS * T;                          // [2T] band magnitudes
+    __half2* SCL = reinterpret_cast<__half2*>(FR + T * SF);  // [NS][T] screen row-axes, start states: (h, h)
+    __half* SCR = reinterpret_cast<__half*>(SCL + NS * T);   // [NS][T] end states
+    uint16_t* list1 = reinterpret_cast<uint16_t*>(FR + T * SF + ((3 * NS * T / 2 + 3) & ~3));  // screened pairs (li << 8 | lj)
+    float* CH = sm;                  // [2T][SC] cost halves, in the place of all of the above once phase 3 is done
+    float* magR = sm + sc_front<M, G, PD>(T, DR);  // [2T] band magnitudes
     float* magF = magR + 2 * T;
-    float* magC = magF + 2 * T;      // [2T] sum of |cost half| per state-side (cost conditioning):
-    float* magC2 = magC + 2 * T;     //      first unit's rows, second unit's rows
+    float* smax = magF + 2 * T;      // [2T] largest row fixed by this state alone
+    float* magC = smax + 2 * T;      // [2T] sum of |cost half| per state-side (cost conditioning):
+    float* magC2 = magC + 2 * T;     //      its two parts
     float* xs = magC2 + 2 * T;       // [2T][XS] centred states
     float* xab = xs + 2 * T * XS;    // [2T][G] per-derivative maxima over the axes
     float* tabs = xab + 2 * T * G;   // two padded duration tables
     float* Ab = tabs + 2 * PT::FLOATS;  // [RMAX][4]: A_r, then b_r
-    uint16_t* list1 = reinterpret_cast<uint16_t*>(Ab + RMAX * 4);  // screened pairs (li << 8 | lj)
-    uint16_t* list2 = list1 + T * T;                                 // feasible pairs
+    float4* box = reinterpret_cast<float4*>(Ab + RMAX * 4);  // [4] per axis: +row (A, b), -row (A, b)
+    uint16_t* list2 = reinterpret_cast<uint16_t*>(box + 4);                                 // feasible pairs
     __shared__ long long s_item;
     __shared__ float s_rown1, s_bmax;
+    __shared__ int s_ng;  // rows left in Ab beside the box rows
+    __shared__ unsigned s_xmax[4];  // largest |derivative c| over the item's states (FP32 bits)
     __shared__ int s_n1[2], s_n2[2];  // list lengths, by duration parity
 
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -1420,10 +1596,6 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
         const int S2 = ni4 + nj4;
         const int r0 = Qd.poly_off[k], nr = Qd.poly_off[k + 1] - r0;
         const long long rg0 = Qd.rowsOff + r0;
-        for (int u = tid; u < nr * 4; u += nthr) {
-            const int r = u >> 2, c = u & 3;
-            Ab[u] = c < M ? P.A32[(rg0 + r) * M + c] : (c == M ? P.bc32[rg0 + r] : 0.f);
-        }
         const int* members = P.members + Qd.listOff + (long long)k * Qd.N;
         float cx[M];
 #pragma unroll
@@ -1443,15 +1615,38 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
             if (hi) stage_state_half<M, G, XS, 1>(Qd.states, P.in_f32, id, valid, cx, xs + row * XS, xab + row * G);
             else stage_state_half<M, G, XS, 0>(Qd.states, P.in_f32, id, valid, cx, xs + row * XS, xab + row * G);
         }
-        if (tid < 32) {  // band scalars of the polytope's rows (warp 0, rows from global memory)
-            float rn = 0.f, bm = 0.f;
-            for (int r = tid; r < nr; r += 32) {
-                float s1 = 0.f;
+        if (tid < 32) {  // the polytope's rows and their band scalars (warp 0; nr <= RMAX < 32)
+            float av[3] = {0.f, 0.f, 0.f}, bv = 0.f, rn = 0.f;
+            if (tid < nr) {
 #pragma unroll
-                for (int a = 0; a < M; ++a) s1 += fabsf(P.A32[(rg0 + r) * M + a]);
-                rn = fmaxf(rn, s1);
-                bm = fmaxf(bm, fabsf(P.bc32[rg0 + r]));
+                for (int a = 0; a < M; ++a) {
+                    av[a] = P.A32[(rg0 + tid) * M + a];
+                    rn += fabsf(av[a]);
+                }
+                bv = P.bc32[rg0 + tid];
             }
+            float bm = fabsf(bv);
+            // the first row along each axis and sign goes to the box (A = 0, b = inf: none), the others to Ab
+            bool boxed = false;
+            if (tid < 4) box[tid] = make_float4(0.f, -NEG_INF, 0.f, -NEG_INF);
+            __syncwarp();
+#pragma unroll
+            for (int sd = 0; sd < 2 * M; ++sd) {
+                const int a = sd >> 1;
+                bool along = tid < nr && ((sd & 1) ? av[a] < 0.f : av[a] > 0.f) && isfinite(av[a]);
+#pragma unroll
+                for (int c = 0; c < M; ++c) along = along && (c == a || av[c] == 0.f);
+                const unsigned m = __ballot_sync(0xffffffffu, along);
+                if (m && tid == __ffs(m) - 1) {
+                    reinterpret_cast<float2*>(box + a)[sd & 1] = make_float2(av[a], bv);
+                    boxed = true;
+                }
+            }
+            const unsigned left = __ballot_sync(0xffffffffu, tid < nr && !boxed);
+            if (tid < nr && !boxed)
+                *reinterpret_cast<float4*>(Ab + 4 * __popc(left & ((1u << tid) - 1u))) =
+                    make_float4(av[0], av[1], M > 2 ? av[2] : bv, M > 2 ? bv : 0.f);
+            if (tid == 0) s_ng = __popc(left);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 rn = fmaxf(rn, __shfl_xor_sync(0xffffffffu, rn, o));
@@ -1470,6 +1665,23 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
         cp_async_wait_all();
         __syncthreads();
 
+        const int lane = tid & 31;
+        {  // every warp finds (and writes) the same maxima
+            unsigned mx[G];
+#pragma unroll
+            for (int c = 0; c < G; ++c) mx[c] = 0u;
+            for (int s = lane; s < S2; s += 32)
+#pragma unroll
+                for (int c = 0; c < G; ++c)
+                    mx[c] = max(mx[c], __float_as_uint(xab[(s < ni4 ? s : T + s - ni4) * G + c]));
+#pragma unroll
+            for (int c = 0; c < G; ++c) {
+                mx[c] = __reduce_max_sync(0xffffffffu, mx[c]);
+                if (lane == 0) s_xmax[c] = mx[c];
+            }
+            __syncwarp();
+        }
+
         const int ngi = ni4 >> 2, ngj = nj4 >> 2;
         const bool act = tid < ngi * ngj;
         const int gi = act ? tid / ngj : 0, gj = act ? tid % ngj : 0;
@@ -1482,32 +1694,48 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                 if (act && li < TI && lj < TJ && i0 + li != j0 + lj) live |= 1u << (qa * 4 + qb);
             }
         for (int t = itc.t0; t < itc.t1; ++t) {
-            // Three block barriers per duration.  The costs of duration t
-            // (phase 4) read only the staged states, table t, the cost
-            // magnitudes and list 2, which duration t+1 rewrites only after
-            // its first barrier (magnitudes in phase 2, the table buffer by the
-            // prefetch for t+2, list 2 in phase 3) -- so duration t+1's halves
-            // overlap the slowest warps' costs of duration t.
+            // Three block barriers per duration, and two more when the costs
+            // are staged.  Costs that are not (phase 4) read only the staged
+            // states, table t and list 2, which duration t+1 rewrites only
+            // after its first barrier (the table buffer by the prefetch for
+            // t+2, list 2 in phase 3) -- so duration t+1's halves overlap
+            // the slowest warps' costs of duration t.
             const int par = (t - itc.t0) & 1;
             const float* tab = tabs + par * PT::FLOATS;
+            // no |row| half exceeds B of this tile and duration: where two
+            // together could leave the FP16 range, the FP16 rows are scaled
+            // by a power of two (short durations; the bands scale with it)
+            float sc = 1.f;
+            {
+                float B = 0.f;
+#pragma unroll
+                for (int c = 0; c < G; ++c)
+                    B = fmaf(tab[PT::ROW_HC * 8 + c] + tab[PT::ROW_HC * 8 + 4 + c], __uint_as_float(s_xmax[c]), B);
+                const int e = (int)(__float_as_uint(B) >> 23) - 127 - 13;  // B < 2^14 2^e
+                if (e > 0) sc = __uint_as_float((unsigned)(127 - min(e, 126)) << 23);
+            }
             // 1. halves: two units per state, each loading the state once --
-            // the first takes reach quads [0, RH), interior points [0, NI/2)
-            // and the band magnitudes, the second the rest
+            // the first takes record quads [0, QH) and the band magnitudes,
+            // the second the rest and the rows fixed by the state alone
             for (int u = tid; u < 2 * S2; u += nthr) {
                 const bool second = u >= S2;
                 const int s = second ? u - S2 : u;
                 const bool right = s >= ni4;
                 const int ls = right ? s - ni4 : s;
+                const int row = (right ? T : 0) + ls;
                 float x[N_];
-                load_state<M, G, PD>(x, xs + (right ? T + ls : ls) * XS);
-                const float* trow = tab + (right ? 4 : 0);
-                float* dU = (right ? UR : UL) + ls * SU;
+                load_state<M, G, PD>(x, xs + row * XS);
+                unsigned* dU = (right ? UR : UL) + ls * SU;
                 void* dS = right ? (void*)SCR : (void*)SCL;
-                float* dF = (right ? FR : FL) + ls * SF;
+                if (second) {
+                    point_halves<M, G, PD>(x, tab, right, (right ? FR : FL) + ls * SF);
+                    smax[row] = single_max<M, G, PD>(x, tab, right);
+                }
+#pragma unroll
+                for (int e = 0; e < N_; ++e) x[e] *= sc;  // the rows are linear in x, and sc is a power of two
                 if (!second) {
-                    reach_quads<M, G, PD, 0, RH>(x, trow, dU, dS, ls, right, T);
-                    point_halves<M, G, PD, 0, NI / 2>(x, tab, right, dF);
-                    const float* xa = xab + (right ? T + ls : ls) * G;
+                    record_quads<M, G, PD, 0, QH>(x, tab, dU, dS, ls, right, T);
+                    const float* xa = xab + row * G;
                     const float* hc = tab + PT::ROW_HC * 8 + (right ? 4 : 0);
                     const float* dc = tab + PT::ROW_DC * 8 + (right ? 4 : 0);
                     float mr = 0.f, md = 0.f;
@@ -1516,11 +1744,10 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                         mr = fmaf(hc[c], xa[c], mr);
                         md = fmaf(dc[c], xa[c], md);
                     }
-                    magR[(right ? T : 0) + ls] = mr;
-                    magF[(right ? T : 0) + ls] = md * s_rown1 + (right ? 0.f : s_bmax);
+                    magR[row] = mr;
+                    magF[row] = md * s_rown1 + (right ? 0.f : s_bmax);
                 } else {
-                    reach_quads<M, G, PD, RH, RQ>(x, trow, dU, dS, ls, right, T);
-                    point_halves<M, G, PD, NI / 2, NI>(x, tab, right, dF);
+                    record_quads<M, G, PD, QH, RQ>(x, tab, dU, dS, ls, right, T);
                 }
             }
             __syncthreads();
@@ -1535,28 +1762,10 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                 s_n1[par ^ 1] = 0;
                 s_n2[par ^ 1] = 0;
             }
-            // the cost rows' magnitudes of this duration (cost conditioning), one
-            // part per unit
-            for (int u = tid; u < 2 * S2; u += nthr) {
-                const bool second = u >= S2;
-                const int s = second ? u - S2 : u;
-                const bool right = s >= ni4;
-                const int ls = right ? s - ni4 : s;
-                float x[N_];
-                load_state<M, G, PD>(x, xs + (right ? T + ls : ls) * XS);
-                using CSG = CostSplit<M, PD, G>;
-                using CS1 = CostSplit<M, PD, 1>;
-                const float mg = DR == G ? (!second ? cost_mag<M, G, PD, G, 0, CSG::FS>(x, tab, right)
-                                                    : cost_mag<M, G, PD, G, CSG::FS, CSG::NP>(x, tab, right))
-                                         : (!second ? cost_mag<M, G, PD, 1, 0, CS1::FS>(x, tab, right)
-                                                    : cost_mag<M, G, PD, 1, CS1::FS, CS1::NP>(x, tab, right));
-                (second ? magC2 : magC)[(right ? T : 0) + ls] = mg;
-            }
-
             // 2. screen and list 1 (positions by a warp prefix of the survivor
             // counts and one shared atomic per warp; the block is whole warps)
             {
-                uint32_t surv = act ? screen_tile<M, G, PD>(T, gi, gj, live, SCL, SCR, magR) : 0u;
+                uint32_t surv = act ? screen_tile<M, G, PD>(T, gi, gj, live, sc, SCL, SCR, magR) : 0u;
                 const int cnt = __popc(surv);
                 int inc = cnt;
 #pragma unroll
@@ -1578,30 +1787,50 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
             // 3. every reach and free row of the screened pairs
             const int n1 = s_n1[par];
             if (tid == 0) nscreened += (unsigned long long)n1;
-            for (int e = tid; e < n1; e += nthr) {
-                const int v = list1[e];
+            const float isc = 1.f / sc;  // exact
+            for (int e0 = tid - lane; e0 < n1; e0 += nthr) {  // whole warps
+                const bool on = e0 + lane < n1;
+                const int v = list1[on ? e0 + lane : e0];
                 const int li = v >> 8, lj = v & 255;
-                const float* ul = UL + li * SU;
-                const float* ur = UR + lj * SU;
-                float r4[4] = {0.f, 0.f, 0.f, 0.f};
+                const uint4* ul = reinterpret_cast<const uint4*>(UL + li * SU);
+                const uint4* ur = reinterpret_cast<const uint4*>(UR + lj * SU);
+                __half2 r2[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) r2[q] = __float2half2_rn(0.f);
 #pragma unroll
                 for (int qd = 0; qd < RQ; ++qd) {
-                    const float4 a = *reinterpret_cast<const float4*>(ul + 4 * qd);
-                    const float4 b = *reinterpret_cast<const float4*>(ur + 4 * qd);
-                    r4[0] = fmaxf(r4[0], fabsf(a.x + b.x));
-                    r4[1] = fmaxf(r4[1], fabsf(a.y + b.y));
-                    r4[2] = fmaxf(r4[2], fabsf(a.z + b.z));
-                    r4[3] = fmaxf(r4[3], fabsf(a.w + b.w));
+                    const uint4 a4 = ul[qd], b4 = ur[qd];
+                    const unsigned av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (4 * qd + j < SS::RW) r2[j] = __hmax2(r2[j], __habs2(__hadd2(as_h2(av[j]), as_h2(bv[j]))));
                 }
-                const float rm = fmaxf(fmaxf(r4[0], r4[1]), fmaxf(r4[2], r4[3]));
-                const float bandR = KR * (magR[li] + magR[T + lj]);
+                const __half2 rr = __hmax2(__hmax2(r2[0], r2[1]), __hmax2(r2[2], r2[3]));
+                float rm = fmaxf(fmaxf(__low2float(rr), __high2float(rr)) * isc, fmaxf(smax[li], smax[T + lj]));
+                const float ms = magR[li] + magR[T + lj], b16 = (KR + KHF) * ms + EH * isc, bandR = KR * ms;
+                // what FP16 leaves open, in FP32: a few pairs one after the
+                // other by the whole warp, many (a warp's pass over one pair
+                // costs about a sixth of a lane's) by their lanes
+                const bool open = on && (!(sc * ms <= MAGH) || !(rm > 1.f + b16 || rm <= 1.f - b16));
+                unsigned am = __ballot_sync(0xffffffffu, open);
+                if (__popc(am) > 6) {
+                    if (open) rm = lane_reach_f32<M, G, PD>(xs + li * XS, xs + (T + lj) * XS, tab);
+                    __syncwarp();
+                } else {
+                    for (; am; am &= am - 1u) {
+                        const int src = __ffs(am) - 1;
+                        const int hv = __shfl_sync(0xffffffffu, v, src);
+                        const float rf = pair_reach_f32<M, G, PD>(xs + (hv >> 8) * XS, xs + (T + (hv & 255)) * XS, tab, lane);
+                        if (lane == src) rm = rf;
+                    }
+                }
                 int outcome = 0;  // 0 certain failure, 1 certainly feasible, 2 ambiguous
-                if (rm <= 1.f + bandR) {
+                if (on && rm <= 1.f + bandR) {
                     const bool rpass = rm <= 1.f - bandR;
                     rp_cnt += rpass ? 1u : 0u;
                     // interior control points P_l = start half + end half, then
                     // every polytope row A_r . P_l - b_r (rows broadcast from Ab)
-                    constexpr int NPQ = (NI * M + 3) / 4;
+                    constexpr int NPQ = SS::NP / 4;
                     const float* pl_ = FL + li * SF;
                     const float* pr_ = FR + lj * SF;
                     float pt[4 * NPQ];
@@ -1615,7 +1844,21 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                         pt[4 * q + 3] = a.w + c.w;
                     }
                     float f2[2] = {NEG_INF, NEG_INF};
-                    for (int r = 0; r < nr; ++r) {
+                    // rows along an axis: A P_la - b is monotone in P_la, so the
+                    // largest value is that of the extreme coordinate
+#pragma unroll
+                    for (int a = 0; a < M; ++a) {
+                        float hi = pt[a], lo = pt[a];
+#pragma unroll
+                        for (int l = 1; l < NI; ++l) {
+                            hi = fmaxf(hi, pt[l * M + a]);
+                            lo = fminf(lo, pt[l * M + a]);
+                        }
+                        const float4 bx = box[a];
+                        f2[0] = fmaxf(f2[0], bx.x * hi - bx.y);
+                        f2[1] = fmaxf(f2[1], bx.z * lo - bx.w);
+                    }
+                    for (int r = 0; r < s_ng; ++r) {
                         const float4 ab = *reinterpret_cast<const float4*>(Ab + r * 4);
                         const float br = M > 2 ? ab.w : ab.z;
 #pragma unroll
@@ -1631,13 +1874,12 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                     if (fm <= bandF) outcome = (rpass && fm <= -bandF) ? 1 : 2;
                 }
                 // list 2 positions: one shared atomic per warp
-                const unsigned am = __activemask();
-                const unsigned fb = __ballot_sync(am, outcome == 1);
+                const unsigned fb = __ballot_sync(0xffffffffu, outcome == 1);
                 if (fb) {
-                    const int lane = tid & 31, leader = __ffs(fb) - 1;
+                    const int leader = __ffs(fb) - 1;
                     int b2 = 0;
                     if (lane == leader) b2 = atomicAdd(&s_n2[par], __popc(fb));
-                    b2 = __shfl_sync(am, b2, leader);
+                    b2 = __shfl_sync(0xffffffffu, b2, leader);
                     if (outcome == 1) list2[b2 + __popc(fb & ((1u << lane) - 1u))] = (uint16_t)v;
                 }
                 if (outcome == 2) append_recheck(P, itd.q, k, i0 + li, j0 + lj, t);
@@ -1646,16 +1888,41 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
             __syncthreads();
 
             const int n2 = s_n2[par];
-            // 4. costs of the feasible pairs from their two staged states (per
-            // segment the sum of squares in row order)
+            // 4. costs of the feasible pairs: many from staged halves, which
+            // take the place of the records, points and list 1, a few from
+            // their two staged states
+            const bool staged = n2 >= SC_STAGE;
+            if (staged) {
+                for (int u = tid; u < 2 * S2; u += nthr) {
+                    const bool second = u >= S2;
+                    const int s = second ? u - S2 : u;
+                    const bool right = s >= ni4;
+                    const int row = right ? T + s - ni4 : s;
+                    float x[N_];
+                    load_state<M, G, PD>(x, xs + row * XS);
+                    using C3 = CostRows<M, PD, G>;
+                    using C1 = CostRows<M, PD, 1>;
+                    const float mg = DR == G ? (!second ? cost_halves<M, G, PD, G, 0, C3::FS>(x, tab, right, CH + row * C3::SC)
+                                                        : cost_halves<M, G, PD, G, C3::FS, C3::NP>(x, tab, right, CH + row * C3::SC))
+                                             : (!second ? cost_halves<M, G, PD, 1, 0, C1::FS>(x, tab, right, CH + row * C1::SC)
+                                                        : cost_halves<M, G, PD, 1, C1::FS, C1::NP>(x, tab, right, CH + row * C1::SC));
+                    (second ? magC2 : magC)[row] = mg;
+                }
+                __syncthreads();
+            }
             for (int e = tid; e < n2; e += nthr) {
                 const int v = list2[e];
-                const int li = v >> 8, lj = v & 255;
-                const float* xi = xs + li * XS;
-                const float* xj = xs + (T + lj) * XS;
-                const float cs = DR == G ? pair_cost_states<M, G, PD, G>(xi, xj, tab)
-                                         : pair_cost_states<M, G, PD, 1>(xi, xj, tab);
-                const float mc = (magC[li] + magC2[li]) + (magC[T + lj] + magC2[T + lj]);
+                const int li = v >> 8, lj = v & 255, rj = T + lj;
+                float cs, mc;
+                if (staged) {
+                    constexpr int SC3 = CostRows<M, PD, G>::SC, SC1 = CostRows<M, PD, 1>::SC;
+                    cs = DR == G ? pair_cost_halves<M, PD, G>(CH + li * SC3, CH + rj * SC3)
+                                 : pair_cost_halves<M, PD, 1>(CH + li * SC1, CH + rj * SC1);
+                    mc = (magC[li] + magC2[li]) + (magC[rj] + magC2[rj]);
+                } else {
+                    cs = DR == G ? pair_cost_states<M, G, PD, G>(xs + li * XS, xs + rj * XS, tab, mc)
+                                 : pair_cost_states<M, G, PD, 1>(xs + li * XS, xs + rj * XS, tab, mc);
+                }
                 if (P.cost64 || mc <= COST_RHO * cs) {  // FP64 models re-cost every edge anyway
                     const long long slot = itd.base + (long long)(i0 + li) * itd.nk + (j0 + lj);
                     atomicOr(&P.resBits[slot], 1u << t);
@@ -1664,6 +1931,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                     append_recheck(P, itd.q, k, i0 + li, j0 + lj, t, true);  // ill-conditioned FP32 cost
                 }
             }
+            if (staged) __syncthreads();  // the next duration's records take the halves' place
         }
     }
     block_add(&P.info->reach_pass, rp_cnt);
@@ -3245,11 +3513,9 @@ size_t smem_one(const BuildParams& P) {
 template <int M, int G, int PD>
 size_t smem_sc(const BuildParams& P) {
     using SS = ScShape<M, G, PD>;
-    const int DR = P.cost_mode == 1 ? 1 : G;
-    const size_t T = (size_t)P.tile;
-    const size_t SF = (size_t)sc_free_stride(Shape<G, PD>::NI, M);
-    size_t f = T * (2 * SS::SU + 2 * SF + 2 * SS::NS + 8) + 2 * T * (SS::XS + G) + 2 * PadTab<G, PD>::FLOATS + RMAX * 4;
-    return f * sizeof(float) + 2 * T * T * sizeof(uint16_t);
+    const int T = P.tile, DR = P.cost_mode == 1 ? 1 : G;
+    const size_t f = (size_t)sc_front<M, G, PD>(T, DR) + 10 * T + 2 * T * (SS::XS + G) + 2 * PadTab<G, PD>::FLOATS + RMAX * 4 + 16;
+    return f * sizeof(float) + T * T * sizeof(uint16_t);
 }
 
 template <int M, int G, int PD>
