@@ -96,6 +96,7 @@ struct plan_ctx {
     int* emitPre = nullptr;
     unsigned long long* recheck = nullptr;
     double* half64 = nullptr;         // FP64 cost halves of every state, duration and side (FP64 cost pass)
+    float* half32 = nullptr;          // FP32 copy behind it (nullptr: no room)
     long long half64Cap = 0;
     // search scratch
     long long capS = -1;
@@ -569,7 +570,11 @@ int prepare(plan_ctx* c, int Q, const plan_query* qs, int max_rows, int shard = 
         const long long need = nrow * (long long)maxT * 2 * c->model.degree * DR * c->model.m;
         if (need > c->half64Cap) {
             if (c->stage_live) cudaEventSynchronize(c->stage_ev);
-            if (!dalloc(c, &c->half64, need)) {
+            // FP64, then an FP32 copy that lets the cost pass skip work (without room for it: all of the work)
+            c->half32 = nullptr;
+            if (dalloc(c, &c->half64, need + (need + 1) / 2)) {
+                c->half32 = reinterpret_cast<float*>(c->half64 + need);
+            } else if (!dalloc(c, &c->half64, need)) {
                 c->half64Cap = 0;
                 return PLAN_ERR_NO_MEMORY;
             }
@@ -644,6 +649,7 @@ int issue(plan_ctx* c) {
     P.cost64 = c->model.arith == PLAN_F64 && !canonical64;
     P.maxT = c->maxT;
     P.half64 = c->half64;
+    P.half32 = c->half32;
     P.max_rows = c->b_max_rows;
     P.tile = (P.arith == PLAN_F64) ? TILE64
              : (P.arith == PLAN_F32) ? (c->tile > 0 ? c->tile : TILE)

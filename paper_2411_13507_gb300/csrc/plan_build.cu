@@ -3309,8 +3309,13 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
 // cheapest duration by the key (cost bits with the low five cleared | t),
 // as the FP64 kernel's slot merge takes it.  The halves depend on one state
 // and one duration only, so k_halves64 computes both halves of every state
-// and duration once (half64 [state][t][side][row]); k_cost64 then adds,
-// squares and takes roots per (edge, duration), one thread per edge.
+// and duration once (half64 [state][t][side][row], an FP32 copy in half32);
+// k_cost64 then adds, squares and takes roots, one thread per edge.  The FP64
+// chain of one duration (PD roots in series on a pipe of two FMA a clock) is
+// what bounds it, and a warp runs as many as its busiest edge has; so FP32
+// costs with an error bound first drop the durations that cannot be the
+// cheapest, mostly all but one (2-D workload, 30,152 edges with 2.7 durations
+// each: 44 -> 24 us).
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256) k_halves64(BuildParams P) {
@@ -3333,8 +3338,50 @@ __global__ void __launch_bounds__(256) k_halves64(BuildParams P) {
 #pragma unroll
         for (int c = 0; c < N_; ++c) x[c] = ldv(Q.states, i * N_ + c, P.in_f32);
         const double* tb = P.tab64 + (long long)(Q.tabOff + t) * L.e_stride;
-        P.half64[u] = half_sum<G>(tb + L.e_C + (d * PD + l) * TG + side * G, x + a, M);
+        const double v = half_sum<G>(tb + L.e_C + (d * PD + l) * TG + side * G, x + a, M);
+        P.half64[u] = v;
+        if (P.half32) P.half32[u] = (float)v;
     }
+}
+
+// Which durations of an edge's mask can be the cheapest in FP64, by their FP32
+// costs.  With S = sum of the halves' magnitudes, rounding the halves and
+// their sum errs by at most 2^-24 (2 S + cost), the norms and the sum of the
+// segments by at most 2^-24 (w + PD + 4) cost for w <= 9 rows a segment and PD
+// <= 7 segments; err = 2^-20 (S + cost) is over twice that for either term and
+// leaves far more than the FP64 key's rounding between a dropped duration and
+// the cheapest one.  A NaN or infinite cost drops nothing.
+template <int M, int PD>
+DEVI uint32_t cheapest_bits(uint32_t bits, const float* hl, const float* hr, int DR) {
+    const int W = DR * M, E = PD * W;
+    uint32_t keep = 0;
+    float ub = __int_as_float(0x7f800000), lb = ub;  // smallest upper bound; smallest lower bound of those kept
+    while (bits) {
+        const int t = __ffs(bits) - 1;
+        bits &= bits - 1u;
+        const float* kl = hl + (long long)t * 2 * E;
+        const float* kr = hr + (long long)t * 2 * E;
+        float cost = 0.f, S = 0.f;
+        for (int l = 0; l < PD; ++l) {
+            float ss = 0.f;
+            for (int w = 0; w < W; ++w) {
+                const float a = kl[l * W + w], b = kr[l * W + w], v = a + b;
+                S += fabsf(a) + fabsf(b);
+                ss = fmaf(v, v, ss);
+            }
+            cost += sqrtf(ss);
+        }
+        const float err = 9.5367431640625e-07f * (S + cost);  // 2^-20
+        if (cost - err > ub) continue;
+        if (cost + err < lb) {  // cheaper than every one kept so far
+            keep = 0;
+            lb = __int_as_float(0x7f800000);
+        }
+        keep |= 1u << t;
+        lb = fminf(lb, cost - err);
+        ub = fminf(ub, cost + err);
+    }
+    return keep;
 }
 
 template <int M, int G, int PD>
@@ -3360,6 +3407,8 @@ __global__ void __launch_bounds__(256) k_cost64(BuildParams P) {
         const double* hi64 = P.half64 + (P.pfxN[q] + i) * per;
         const double* hj64 = P.half64 + (P.pfxN[q] + j) * per;
         uint32_t bits = Q.mask[e];
+        if (P.half32 && (bits & (bits - 1u)))
+            bits = cheapest_bits<M, PD>(bits, P.half32 + (P.pfxN[q] + i) * per, P.half32 + (P.pfxN[q] + j) * per + E, DR);
         unsigned long long best = KEY_NONE;
         while (bits) {
             const int t = __ffs(bits) - 1;

@@ -143,6 +143,7 @@ struct BuildParams {
     int cost64;                // FP64 model on the FP32 pair kernels: canonical FP64 cost pass after compaction
     int maxT;                  // most durations of any query
     double* half64;            // [totN][maxT][2][p * DR * m] FP64 cost halves (FP64 cost pass)
+    float* half32;             // the same in FP32, or nullptr
     double eps;
     const QueryDesc* qd;       // [Q]
     const long long* pfxMask;  // [Q+1] prefix of N*W        (membership threads)
