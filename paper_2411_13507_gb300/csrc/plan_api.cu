@@ -4,6 +4,8 @@
 // that plan_wait reads.  No exception crosses the ABI.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1443,6 +1445,8 @@ int plan_prepare_search_batched(plan_ctx* c, int Q, const plan_search_query* qs)
         tot += in.N;
         if (in.N > maxN) maxN = in.N;
     }
+    // the largest first: the batch ends with its longest query
+    std::stable_sort(hq.begin(), hq.end(), [](const SearchQueryDesc& a, const SearchQueryDesc& b) { return a.N > b.N; });
     if (tot > c->capS) {
         if (!dalloc(c, &c->sdist, tot) || !dalloc(c, &c->sbest, tot) || !dalloc(c, &c->spred, tot) ||
             !dalloc(c, &c->sfront, 2LL * tot))
@@ -1491,6 +1495,7 @@ int plan_search_batched(plan_ctx* c) {
     B.in_f32 = c->model.input == PLAN_IN_F32;
     B.w_f64 = c->model.arith == PLAN_F64;
     B.max_sweeps = c->max_sweeps > 0 ? c->max_sweeps : c->sMaxN + 1;
+    B.maxN = c->sMaxN;
     B.qd = c->d_sqd;
     B.dist = c->sdist;
     B.bestU = c->sbest;

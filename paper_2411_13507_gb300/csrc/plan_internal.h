@@ -239,7 +239,7 @@ struct SearchQueryDesc {
 };
 
 struct BatchSearchParams {
-    int Q, m, n, in_f32, w_f64, max_sweeps;
+    int Q, m, n, in_f32, w_f64, max_sweeps, maxN;
     const SearchQueryDesc* qd;
     unsigned long long* dist;
     unsigned long long* bestU;

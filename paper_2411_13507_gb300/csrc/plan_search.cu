@@ -477,133 +477,200 @@ __global__ void __launch_bounds__(1024, 1) k_search(SearchParams P) {
 }
 
 // ---------------------------------------------------------------------------
-// Batched search: one 1024-thread CTA per query; the same phases as k_search
-// with block barriers in place of the grid barrier.  Per-query status: OK,
-// NO_PATH (path_len 0, cost +inf), CAPACITY (path longer than path_cap;
-// path_len = the length needed), TIMEOUT (sweep bound), INVALID_ARG.
+// Batched search: one thread-block cluster per query; the same phases as
+// k_search with cluster barriers in place of the grid barrier.  Per-query
+// status: OK, NO_PATH (path_len 0, cost +inf), CAPACITY (path longer than
+// path_cap; path_len = the length needed), TIMEOUT (sweep bound), INVALID_ARG.
+//
+// A sweep is a chain of L2 round trips per frontier vertex (its edges, then
+// the relaxing atomics), so a query's time is its vertices per warp times that
+// latency, and the largest query's is the batch's: a CTA per 1024 vertices, up
+// to 8 of a cluster, shortens it, and four groups of 32 edges are in flight at
+// once (256 queries of 512 to 16,384 vertices, 125 M edges: one CTA a query
+// and one group 6.55 ms, now 1.95 ms).  CTAs a small query does not need leave at
+// once; barriers count the threads that have not left.
 // ---------------------------------------------------------------------------
+constexpr int SB_CLUSTER = 8, SB_VERTICES = 1024;
+
+// The out-edges of v by a warp: f(u, w) with the targets (-1: none) and
+// weights of four groups of 32 edges, loaded before any is used.
+template <typename F>
+DEVI void each_edge(const SearchQueryDesc& Q, int w_f64, int N, int v, int lane, F f) {
+    const long long e0 = Q.row_off[v], e1 = Q.row_off[v + 1];
+    for (long long eb = e0; eb < e1; eb += 128) {
+        int u[4];
+        double w[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const long long e = eb + 32 * c + lane;
+            u[c] = e < e1 ? Q.col[e] : -1;
+            w[c] = e < e1 ? (w_f64 ? ((const double*)Q.w)[e] : (double)((const float*)Q.w)[e]) : 0.0;
+        }
+        f(u, w);
+    }
+}
+
 __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
-    const SearchQueryDesc& Q = B.qd[blockIdx.x];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const SearchQueryDesc& Q = B.qd[blockIdx.x / cluster.num_blocks()];
     const int N = Q.N;
+    // CTAs of this query; the others leave (bad queries need none beyond the first)
+    const int nc = min((int)cluster.num_blocks(), (N + SB_VERTICES - 1) / SB_VERTICES > 1 ? (N + SB_VERTICES - 1) / SB_VERTICES : 1);
+    const int rank = (int)cluster.block_rank();
+    if (rank >= nc) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int v0 = rank * (int)blockDim.x + tid, vstep = nc * (int)blockDim.x;   // this thread's vertices
+    const int w0 = wid * nc + rank, wstep = nc * nw;                            // this warp's vertices
     unsigned long long* dist = B.dist + Q.off;
     unsigned long long* best = B.bestU + Q.off;
     int* pred = B.pred + Q.off;
     unsigned char* front = B.front + 2 * Q.off;
-    __shared__ unsigned long long s_nd[2];
-    __shared__ int s_id[2];
-    __shared__ int s_changed;
-    __shared__ int s_bad;
+    __shared__ unsigned long long s_wd[2][32];
+    __shared__ int s_wi[2][32];
+    __shared__ unsigned long long s_nd[2][SB_CLUSTER];  // rank 0's: every CTA's nearest start and goal
+    __shared__ int s_id[2][SB_CLUSTER];
+    __shared__ int s_changed[3];                        // rank 0's: a CTA changed a distance, by sweep mod 3
+    __shared__ int s_bad, s_any;
     if (tid == 0) {
-        s_nd[0] = s_nd[1] = ~0ull;
-        s_id[0] = s_id[1] = 0x7fffffff;
-        s_bad = 0;
         const long long E = *Q.count;
-        if (N < 1 || E < 0 || E > Q.cap) s_bad = 1;
+        s_bad = N < 1 || E < 0 || E > Q.cap;
+        s_changed[0] = s_changed[1] = s_changed[2] = 0;
+        s_any = 0;
     }
-    for (int v = tid; v < N; v += blockDim.x) {
+    // initial values; the nearest vertices of start and goal (ties to the lowest id)
+    unsigned long long kb[2] = {~0ull, ~0ull};
+    int ki[2] = {0x7fffffff, 0x7fffffff};
+    for (int v = v0; v < N; v += vstep) {
         dist[v] = DINF;
         best[v] = ~0ull;
         pred[v] = 0x7fffffff;
         front[v] = 0;
         front[N + v] = 0;
+        double ds = 0.0, dg = 0.0;
+        for (int a = 0; a < B.m; ++a) {
+            const double x = ldd(Q.states, (long long)v * B.n + a, B.in_f32);
+            const double ts = __dsub_rn(x, Q.start[a]);
+            const double tg = __dsub_rn(x, Q.goal[a]);
+            ds = __dadd_rn(ds, __dmul_rn(ts, ts));
+            dg = __dadd_rn(dg, __dmul_rn(tg, tg));
+        }
+        keep_min(kb[0], ki[0], (unsigned long long)__double_as_longlong(ds), v);
+        keep_min(kb[1], ki[1], (unsigned long long)__double_as_longlong(dg), v);
     }
-    __syncthreads();
-    if (s_bad) {
-        if (tid == 0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long ob = __shfl_xor_sync(0xffffffffu, kb[q], o);
+            const int oi = __shfl_xor_sync(0xffffffffu, ki[q], o);
+            keep_min(kb[q], ki[q], ob, oi);
+        }
+        if (lane == 0) {
+            s_wd[q][wid] = kb[q];
+            s_wi[q][wid] = ki[q];
+        }
+    }
+    cluster.sync();  // every CTA of the query runs: rank 0's shared memory can be written
+    if (s_bad) {     // the same in all of them
+        if (tid == 0 && rank == 0) {
             *Q.status = PLAN_ERR_INVALID_ARG;
             if (N >= 1) *Q.path_len = 0;
         }
         return;
     }
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int v = tid; v < N; v += blockDim.x) {
-            double ds = 0.0, dg = 0.0;
-            for (int a = 0; a < B.m; ++a) {
-                const double x = ldd(Q.states, (long long)v * B.n + a, B.in_f32);
-                const double ts = __dsub_rn(x, Q.start[a]);
-                const double tg = __dsub_rn(x, Q.goal[a]);
-                ds = __dadd_rn(ds, __dmul_rn(ts, ts));
-                dg = __dadd_rn(dg, __dmul_rn(tg, tg));
-            }
-            const unsigned long long bs = (unsigned long long)__double_as_longlong(ds);
-            const unsigned long long bg = (unsigned long long)__double_as_longlong(dg);
-            if (pass == 0) {
-                atomicMin(&s_nd[0], bs);
-                atomicMin(&s_nd[1], bg);
-            } else {
-                if (bs == s_nd[0]) atomicMin(&s_id[0], v);
-                if (bg == s_nd[1]) atomicMin(&s_id[1], v);
-            }
-        }
-        __syncthreads();
+    if (tid < 2) {
+        unsigned long long b = ~0ull;
+        int i = 0x7fffffff;
+        for (int w = 0; w < nw; ++w) keep_min(b, i, s_wd[tid][w], s_wi[tid][w]);
+        *cluster.map_shared_rank(&s_nd[tid][rank], 0) = b;
+        *cluster.map_shared_rank(&s_id[tid][rank], 0) = i;
     }
-    const int s = s_id[0], g = s_id[1];
-    if (tid == 0) {
+    cluster.sync();
+    int sg[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        unsigned long long b = ~0ull;
+        sg[q] = 0x7fffffff;
+        const unsigned long long* nd = cluster.map_shared_rank(&s_nd[q][0], 0);
+        const int* id = cluster.map_shared_rank(&s_id[q][0], 0);
+        for (int r = 0; r < nc; ++r) keep_min(b, sg[q], nd[r], id[r]);
+    }
+    const int s = sg[0], g = sg[1];
+    if (tid == 0 && rank == 0) {
         dist[s] = 0ull;
         front[s] = 1;
     }
+    cluster.sync();
+    int* changed0 = cluster.map_shared_rank(&s_changed[0], 0);
     int cur = 0, it = 0;
     volatile unsigned long long* vdist = dist;
     for (;;) {
-        if (tid == 0) s_changed = 0;
-        __syncthreads();
+        // the slot of the next sweep: last read before the barrier that ended the sweep before this one
+        if (tid == 0 && rank == 0) s_changed[(it + 1) % 3] = 0;
         bool my_change = false;
         const unsigned long long gd = vdist[g];   // vertices not closer than the goal do not relax
-        for (int v = wid; v < N; v += nw) {
+        for (int v = w0; v < N; v += wstep) {
             if (!front[cur * N + v]) continue;
             __syncwarp();
             if (lane == 0) front[cur * N + v] = 0;
             if (vdist[v] >= gd) continue;
             const double dv = __longlong_as_double((long long)vdist[v]);
-            const long long e0 = Q.row_off[v], e1 = Q.row_off[v + 1];
-            for (long long e = e0 + lane; e < e1; e += 32) {
-                const int u = Q.col[e];
-                if (u < 0 || u >= N) continue;
-                const double w = B.w_f64 ? ((const double*)Q.w)[e] : (double)((const float*)Q.w)[e];
-                const unsigned long long nd = (unsigned long long)__double_as_longlong(__dadd_rn(dv, w));
-                const unsigned long long old = atomicMin(&dist[u], nd);
-                if (nd < old) {
-                    front[(cur ^ 1) * N + u] = 1;
-                    my_change = true;
+            each_edge(Q, B.w_f64, N, v, lane, [&](const int (&u)[4], const double (&w)[4]) {
+                unsigned long long nd[4], old[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    nd[c] = (unsigned long long)__double_as_longlong(__dadd_rn(dv, w[c]));
+                    old[c] = u[c] >= 0 && u[c] < N ? atomicMin(&dist[u[c]], nd[c]) : 0ull;
                 }
-            }
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (nd[c] < old[c]) {
+                        front[(cur ^ 1) * N + u[c]] = 1;
+                        my_change = true;
+                    }
+            });
         }
-        if (__any_sync(0xffffffffu, my_change) && lane == 0) s_changed = 1;
+        if (my_change) s_any = 1;
         __syncthreads();
-        const int ch = s_changed;
+        if (tid == 0 && s_any) {
+            changed0[it % 3] = 1;
+            s_any = 0;
+        }
+        cluster.sync();
+        const int ch = changed0[it % 3];
         ++it;
         if (!ch) break;
         if (it > B.max_sweeps) {
-            if (tid == 0) {
+            if (tid == 0 && rank == 0) {
                 *Q.status = PLAN_ERR_TIMEOUT;
                 *Q.path_len = 0;
             }
+            cluster.sync();  // rank 0's shared memory has been read
             return;
         }
         cur ^= 1;
-        __syncthreads();
     }
     const unsigned long long dgoal = vdist[g];
     for (int pass = 0; pass < 2; ++pass) {
-        for (int v = wid; v < N; v += nw) {
+        for (int v = w0; v < N; v += wstep) {
             const unsigned long long dvb = vdist[v];
             if (dvb >= dgoal) continue;   // only vertices closer than the goal can precede path vertices
             const double dv = __longlong_as_double((long long)dvb);
-            const long long e0 = Q.row_off[v], e1 = Q.row_off[v + 1];
-            for (long long e = e0 + lane; e < e1; e += 32) {
-                const int u = Q.col[e];
-                if (u < 0 || u >= N || u == s) continue;
-                const double w = B.w_f64 ? ((const double*)Q.w)[e] : (double)((const float*)Q.w)[e];
-                const unsigned long long nd = (unsigned long long)__double_as_longlong(__dadd_rn(dv, w));
-                if (nd != vdist[u]) continue;
-                if (pass == 0) atomicMin(&best[u], dvb);
-                else if (best[u] == dvb) atomicMin(&pred[u], v);
-            }
+            each_edge(Q, B.w_f64, N, v, lane, [&](const int (&u)[4], const double (&w)[4]) {
+                unsigned long long du[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) du[c] = u[c] >= 0 && u[c] < N && u[c] != s ? vdist[u[c]] : ~0ull;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if ((unsigned long long)__double_as_longlong(__dadd_rn(dv, w[c])) != du[c]) continue;
+                    if (pass == 0) atomicMin(&best[u[c]], dvb);
+                    else if (best[u[c]] == dvb) atomicMin(&pred[u[c]], v);
+                }
+            });
         }
-        __syncthreads();
+        cluster.sync();
     }
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
         const unsigned long long dg = vdist[g];
         int st = PLAN_OK;
         if (dg >= DINF) {
@@ -1432,9 +1499,21 @@ int launch_search_to(const GoalSearchParams& G, void* stream, int num_sms, int* 
 
 int launch_search_batched(const BatchSearchParams& P, void* stream, int* launches) {
     if (P.Q <= 0) return 0;
-    k_search_batched<<<P.Q, 1024, 0, (cudaStream_t)stream>>>(P);
+    int C = 1;  // CTAs a query: what the largest one takes
+    while (C < SB_CLUSTER && (long long)C * SB_VERTICES < P.maxN) C *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)P.Q * C);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     ++*launches;
-    return (int)cudaGetLastError();
+    return (int)cudaLaunchKernelEx(&cfg, k_search_batched, P);
 }
 
 int launch_search(const SearchParams& P, void* stream, int num_sms, int* launches) {
