@@ -123,14 +123,14 @@ PDEV void unit_row(const PlanesParams& Q, int r0, int r, double* n, double& c) {
     c = pld64(Q.b, r0 + r, Q.in_f32) * rn;
 }
 
-// One warp per obstacle: faces (unit normal, offset) and edges, compacted;
-// FP64, rounded to FP32 at the end.  Edge record (4 float4): base point and
+// One warp per obstacle (3-D): faces (unit normal, offset) and edges,
+// compacted; FP64, rounded to FP32 at the end.  Edge record (4 float4): base point and
 // t_lo; unit direction and t_hi; then in 2-D the unit normals of the rows
 // that end the segment at t_lo and t_hi (zero at an infinite end) and the
 // edge's own unit normal and offset, in 3-D the unit normals of its two
 // facets.
-template <int M>
 __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
+    constexpr int M = 3;
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
             }
             face[r] = f;
         }
-        // edges: a facet's line (2-D) or a pair of facets' line (3-D)
-        const int ncand = M == 2 ? nr : nr * nr;
+        // edges: a pair of facets' line
+        const int ncand = nr * nr;
         int count = 0;
         for (int c0 = 0; c0 < ncand; c0 += 32) {
             const int c = c0 + lane;
@@ -165,49 +165,34 @@ __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
             double z0[3] = {0.0, 0.0, 0.0}, d[3] = {0.0, 0.0, 0.0}, tlo = 0.0, thi = 0.0;
             int ra = -1, rb = -1, rlo = -1, rhi = -1;  // the edge's own facets, the rows at its ends
             if (c < ncand) {
-                if (M == 2) {
-                    const double a0 = pld64(Q.A, (long long)(r0 + c) * 2, Q.in_f32);
-                    const double a1 = pld64(Q.A, (long long)(r0 + c) * 2 + 1, Q.in_f32);
-                    const double n2 = a0 * a0 + a1 * a1;
-                    if (n2 > 0.0) {
-                        const double rn = 1.0 / sqrt(n2), bb = pld64(Q.b, r0 + c, Q.in_f32);
-                        d[0] = -a1 * rn;
-                        d[1] = a0 * rn;
-                        z0[0] = a0 * bb / n2;   // the line's point nearest the origin
-                        z0[1] = a1 * bb / n2;
-                        ra = c;
-                        ok = true;
+                const int r1 = c / nr, r2 = c - r1 * nr;
+                if (r1 < r2) {
+                    double a[3], bq[3], b1, b2;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        a[k] = pld64(Q.A, (long long)(r0 + r1) * 3 + k, Q.in_f32);
+                        bq[k] = pld64(Q.A, (long long)(r0 + r2) * 3 + k, Q.in_f32);
                     }
-                } else {
-                    const int r1 = c / nr, r2 = c - r1 * nr;
-                    if (r1 < r2) {
-                        double a[3], bq[3], b1, b2;
+                    b1 = pld64(Q.b, r0 + r1, Q.in_f32);
+                    b2 = pld64(Q.b, r0 + r2, Q.in_f32);
+                    double x[3] = {a[1] * bq[2] - a[2] * bq[1], a[2] * bq[0] - a[0] * bq[2], a[0] * bq[1] - a[1] * bq[0]};
+                    const double xx = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
+                    const double aa = a[0] * a[0] + a[1] * a[1] + a[2] * a[2];
+                    const double bbq = bq[0] * bq[0] + bq[1] * bq[1] + bq[2] * bq[2];
+                    if (xx > 1e-20 * aa * bbq) {
+                        // z0 = alpha a + beta bq with a . z0 = b1, bq . z0 = b2
+                        const double ab = a[0] * bq[0] + a[1] * bq[1] + a[2] * bq[2];
+                        const double det = aa * bbq - ab * ab;
+                        const double al = (b1 * bbq - b2 * ab) / det, be = (b2 * aa - b1 * ab) / det;
+                        const double rx = 1.0 / sqrt(xx);
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            a[k] = pld64(Q.A, (long long)(r0 + r1) * 3 + k, Q.in_f32);
-                            bq[k] = pld64(Q.A, (long long)(r0 + r2) * 3 + k, Q.in_f32);
+                            z0[k] = al * a[k] + be * bq[k];
+                            d[k] = x[k] * rx;
                         }
-                        b1 = pld64(Q.b, r0 + r1, Q.in_f32);
-                        b2 = pld64(Q.b, r0 + r2, Q.in_f32);
-                        double x[3] = {a[1] * bq[2] - a[2] * bq[1], a[2] * bq[0] - a[0] * bq[2], a[0] * bq[1] - a[1] * bq[0]};
-                        const double xx = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
-                        const double aa = a[0] * a[0] + a[1] * a[1] + a[2] * a[2];
-                        const double bbq = bq[0] * bq[0] + bq[1] * bq[1] + bq[2] * bq[2];
-                        if (xx > 1e-20 * aa * bbq) {
-                            // z0 = alpha a + beta bq with a . z0 = b1, bq . z0 = b2
-                            const double ab = a[0] * bq[0] + a[1] * bq[1] + a[2] * bq[2];
-                            const double det = aa * bbq - ab * ab;
-                            const double al = (b1 * bbq - b2 * ab) / det, be = (b2 * aa - b1 * ab) / det;
-                            const double rx = 1.0 / sqrt(xx);
-#pragma unroll
-                            for (int k = 0; k < 3; ++k) {
-                                z0[k] = al * a[k] + be * bq[k];
-                                d[k] = x[k] * rx;
-                            }
-                            ra = r1;
-                            rb = r2;
-                            ok = true;
-                        }
+                        ra = r1;
+                        rb = r2;
+                        ok = true;
                     }
                 }
                 if (ok) {
@@ -222,24 +207,137 @@ __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
                 ed[0] = make_float4((float)z0[0], (float)z0[1], (float)z0[2], __double2float_rd(tlo));
                 ed[1] = make_float4((float)d[0], (float)d[1], (float)d[2], __double2float_ru(thi));
                 double na[3], nb[3], ca = 0.0, cb = 0.0;
-                if (M == 2) {
-                    // the normals of the rows at the two ends (zero at an infinite end), own normal and offset
-                    double nl[3] = {0.0, 0.0, 0.0}, nh[3] = {0.0, 0.0, 0.0}, cl = 0.0, ch = 0.0;
-                    if (rlo >= 0) unit_row<M>(Q, r0, rlo, nl, cl);
-                    if (rhi >= 0) unit_row<M>(Q, r0, rhi, nh, ch);
-                    unit_row<M>(Q, r0, ra, na, ca);
-                    ed[2] = make_float4((float)nl[0], (float)nl[1], (float)nh[0], (float)nh[1]);
-                    ed[3] = make_float4((float)na[0], (float)na[1], (float)ca, 0.f);
-                } else {
-                    unit_row<M>(Q, r0, ra, na, ca);
-                    unit_row<M>(Q, r0, rb, nb, cb);
-                    ed[2] = make_float4((float)na[0], (float)na[1], (float)na[2], 0.f);
-                    ed[3] = make_float4((float)nb[0], (float)nb[1], (float)nb[2], 0.f);
+                unit_row<M>(Q, r0, ra, na, ca);
+                unit_row<M>(Q, r0, rb, nb, cb);
+                ed[2] = make_float4((float)na[0], (float)na[1], (float)na[2], 0.f);
+                ed[3] = make_float4((float)nb[0], (float)nb[1], (float)nb[2], 0.f);
+            }
+            count += __popc(bal);
+        }
+        if (lane == 0) {
+            Q.nedge[o] = count < Q.max_edges ? count : Q.max_edges;
+            if (count > Q.max_edges) p_status(Q.info, PLAN_ERR_UNSUPPORTED, DET_ROWS);
+        }
+    }
+}
+
+// The turn from an edge's normal a to the normal n of the row that ends it: its
+// sign, or NaN where they do not span a cone (no row there, or parallel).
+PDEV float turn(float ax, float ay, float nx, float ny) {
+    const float kk = ax * ny - ay * nx;
+    return kk > 0.f ? 1.f : (kk < 0.f ? -1.f : __int_as_float(0x7fc00000));
+}
+
+// The 2-D form of k_planes_prep and k_planes_geom in one launch: one warp per
+// obstacle, four lanes per row (its line's clipping against the other rows and
+// the three unit normals split over them), eight rows at a time.  A chain of
+// FP64 instructions on a pipe that takes about 64 cycles for each of a warp's,
+// so what counts is their number a lane: divisions by 2 rows instead of 7,
+// one root instead of three (500 obstacles: 2.6 + 19 -> 12 us).
+__global__ void __launch_bounds__(128) k_planes_geom2(PlanesParams Q) {
+    const int lane = threadIdx.x & 31, rs = lane & 3;
+    const double inf = __longlong_as_double(0x7FF0000000000000ll);
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long o = gw; o < Q.n_obst; o += nw) {
+        const int r0 = Q.obst_off[o];
+        int nr = Q.obst_off[o + 1] - r0;
+        if (nr < 0 || nr > Q.max_orows || r0 < 0 || (nr > 0 && (!Q.A || !Q.b))) {
+            if (lane == 0) p_status(Q.info, nr > Q.max_orows ? PLAN_ERR_UNSUPPORTED : PLAN_ERR_INVALID_ARG, DET_ROWS);
+            nr = 0;
+        }
+        float4* row = reinterpret_cast<float4*>(Q.orow) + o * Q.max_orows;
+        float4* face = reinterpret_cast<float4*>(Q.face) + o * Q.max_orows;
+        float4* edge = reinterpret_cast<float4*>(Q.edge) + EDGE_F4 * o * Q.max_edges;
+        for (int r = nr + lane; r < Q.max_orows; r += 32) face[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        int count = 0;
+        for (int c0 = 0; c0 < nr; c0 += 8) {
+            const int c = c0 + (lane >> 2);
+            bool ok = false;
+            double z0[2] = {0.0, 0.0}, d[2] = {0.0, 0.0}, tlo = -inf, thi = inf;
+            int rlo = -1, rhi = -1;
+            if (c < nr) {
+                const double a0 = pld64(Q.A, (long long)(r0 + c) * 2, Q.in_f32);
+                const double a1 = pld64(Q.A, (long long)(r0 + c) * 2 + 1, Q.in_f32);
+                const double n2 = a0 * a0 + a1 * a1;
+                if (rs == 0)
+                    row[c] = make_float4(pld32(Q.A, (long long)(r0 + c) * 2, Q.in_f32),
+                                         pld32(Q.A, (long long)(r0 + c) * 2 + 1, Q.in_f32), 0.f, pld32(Q.b, r0 + c, Q.in_f32));
+                if (n2 > 0.0) {
+                    const double rn = 1.0 / sqrt(n2), bb = pld64(Q.b, r0 + c, Q.in_f32);
+                    d[0] = -a1 * rn;
+                    d[1] = a0 * rn;
+                    z0[0] = a0 * bb / n2;   // the line's point nearest the origin
+                    z0[1] = a1 * bb / n2;
+                    ok = true;
+                    for (int r = rs; r < nr; r += 4) {
+                        double ad = 0.0, az = 0.0;
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) {
+                            const double A = pld64(Q.A, (long long)(r0 + r) * 2 + a, Q.in_f32);
+                            ad = fma(A, d[a], ad);
+                            az = fma(A, z0[a], az);
+                        }
+                        const double b = pld64(Q.b, r0 + r, Q.in_f32), slack = b - az;
+                        if (fabs(ad) <= 1e-12) {
+                            if (slack < -1e-12 * (fabs(b) + 1.0)) {  // parallel to the line and excluding it
+                                tlo = inf;
+                                thi = -inf;
+                            }
+                        } else {
+                            const double t = slack / ad;
+                            if (ad > 0.0) {
+                                if (t < thi) {
+                                    thi = t;
+                                    rhi = r;
+                                }
+                            } else if (t > tlo) {
+                                tlo = t;
+                                rlo = r;
+                            }
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int of = 1; of < 4; of <<= 1) {  // the four lanes' intervals; ties to the lower row, as in row order
+                const double l2 = __shfl_xor_sync(0xffffffffu, tlo, of), h2 = __shfl_xor_sync(0xffffffffu, thi, of);
+                const int rl2 = __shfl_xor_sync(0xffffffffu, rlo, of), rh2 = __shfl_xor_sync(0xffffffffu, rhi, of);
+                if (l2 > tlo || (l2 == tlo && (unsigned)rl2 < (unsigned)rlo)) {
+                    tlo = l2;
+                    rlo = rl2;
+                }
+                if (h2 < thi || (h2 == thi && (unsigned)rh2 < (unsigned)rhi)) {
+                    thi = h2;
+                    rhi = rh2;
+                }
+            }
+            ok = ok && tlo <= thi;
+            const unsigned bal = __ballot_sync(0xffffffffu, ok && rs == 0);
+            const int slot = count + __popc(bal & ((1u << (lane & ~3)) - 1u));
+            // unit normals: lane 0 of the four the row's own, 1 and 2 of the rows at its ends (zero at an infinite end)
+            double n[3] = {0.0, 0.0, 0.0}, cn = 0.0;
+            const int rn_ = rs == 0 ? c : (rs == 1 ? rlo : rhi);
+            if (c < nr && rs < 3 && rn_ >= 0) unit_row<2>(Q, r0, rn_, n, cn);
+            const float nx = (float)n[0], ny = (float)n[1];
+            const float hx = __shfl_down_sync(0xffffffffu, nx, 1), hy = __shfl_down_sync(0xffffffffu, ny, 1);
+            const float lx = hx, ly = hy;  // in lane 0 of the four: the normals at t_lo, t_hi
+            const float gx = __shfl_down_sync(0xffffffffu, nx, 2), gy = __shfl_down_sync(0xffffffffu, ny, 2);
+            if (c < nr && rs == 0) face[c] = make_float4(nx, ny, 0.f, (float)cn);
+            if (ok && slot < Q.max_edges) {
+                float4* ed = edge + EDGE_F4 * slot;
+                if (rs == 0) {
+                    ed[0] = make_float4((float)z0[0], (float)z0[1], turn(nx, ny, lx, ly), __double2float_rd(tlo));
+                    ed[1] = make_float4((float)d[0], (float)d[1], turn(nx, ny, gx, gy), __double2float_ru(thi));
+                    ed[3] = make_float4(nx, ny, (float)cn, 0.f);
+                } else if (rs == 1) {
+                    ed[2] = make_float4(nx, ny, hx, hy);
                 }
             }
             count += __popc(bal);
         }
         if (lane == 0) {
+            Q.ocount[o] = nr;
             Q.nedge[o] = count < Q.max_edges ? count : Q.max_edges;
             if (count > Q.max_edges) p_status(Q.info, PLAN_ERR_UNSUPPORTED, DET_ROWS);
         }
@@ -293,6 +391,187 @@ __global__ void __launch_bounds__(256) k_planes_ub(PlanesParams Q) {
             if (lane == 0) atomicMin(reinterpret_cast<unsigned*>(Q.ub) + p, ub);
         } else if (act && ub != 0x7f7f7f7fu) {
             atomicMin(reinterpret_cast<unsigned*>(Q.ub) + p, ub);
+        }
+    }
+}
+
+// One obstacle's rows, faces and edges: in global memory, or (SH) in shared
+// memory with `stride` float4 from one entry of an obstacle to its next.
+template <bool SH>
+struct Geom {
+    const float4 *rows, *faces, *edges;
+    int stride, nr, ne;
+    PDEV float4 at(const float4* p, int i) const { return SH ? p[i * stride] : __ldg(p + i); }
+    PDEV float4 row(int r) const { return at(rows, r); }
+    PDEV float4 face_of(int r) const { return at(faces, r); }
+    PDEV float4 edge_of(int e, int i) const { return at(edges, EDGE_F4 * e + i); }
+};
+
+// The point z of a 2-D obstacle nearest to each of NP points v, and its
+// squared distance (0 and v itself inside; infinite without an edge): the
+// first edge segment that holds it by sign tests, else the nearest candidate.
+// A segment whose parameter needs no clamping and whose facet v lies outside of
+// holds the projection; a vertex does when v - vertex lies in the cone of its
+// two facet normals.  Without a branch: the lanes of a warp (one obstacle
+// each) settle on different edges, so every edge is run anyway.
+template <bool SH, int NP>
+PDEV void closest_2d(const float (&v)[NP][2], const Geom<SH>& geo, float (&z)[NP][2], float (&d2)[NP]) {
+    const float inf = __int_as_float(0x7f800000);
+    bool in[NP], found[NP];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) in[i] = true;
+    for (int r = 0; r < geo.nr; ++r) {
+        const float4 f = geo.row(r);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) in[i] = in[i] & (pdot<2>(f, v[i]) - f.w <= 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        z[i][0] = v[i][0];
+        z[i][1] = v[i][1];
+        d2[i] = in[i] ? 0.f : inf;
+        found[i] = in[i];
+    }
+    for (int e = 0; e < geo.ne; ++e) {
+        const float4 e0 = geo.edge_of(e, 0), e1 = geo.edge_of(e, 1), e2 = geo.edge_of(e, 2), e3 = geo.edge_of(e, 3);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            float t = e1.x * (v[i][0] - e0.x);
+            t = fmaf(e1.y, v[i][1] - e0.y, t);
+            const float tc = fminf(fmaxf(t, e0.w), e1.w);
+            const float cx = fmaf(tc, e1.x, e0.x), cy = fmaf(tc, e1.y, e0.y);
+            const float wx = v[i][0] - cx, wy = v[i][1] - cy;
+            const float dd = fmaf(wy, wy, wx * wx);
+            const float sd = fmaf(e3.y, v[i][1], e3.x * v[i][0]) - e3.z;  // outside this facet?
+            // a clamped end: v - c in the cone of the two normals, whose turn sg is (NaN: no vertex there)
+            const bool lo = t < e0.w;
+            const float nx = lo ? e2.x : e2.z, ny = lo ? e2.y : e2.w, sg = lo ? e0.z : e1.z;
+            const bool cone = ((e3.x * wy - e3.y * wx) * sg >= 0.f) & ((wx * ny - wy * nx) * sg >= 0.f);
+            const bool hit = tc == t ? sd > 0.f : cone;
+            const bool take = !found[i] & (hit | (dd < d2[i]));
+            found[i] |= hit;
+            if (take) {
+                d2[i] = dd;
+                z[i][0] = cx;
+                z[i][1] = cy;
+            }
+        }
+    }
+}
+
+// The point z of the obstacle nearest to v and its squared distance (0 and v
+// itself inside; infinite for an obstacle without a face or an edge).
+template <int M, bool SH>
+PDEV void pair_closest(const float (&v)[M], const Geom<SH>& geo, float (&z)[M], float& d2) {
+    const float inf = __int_as_float(0x7f800000);
+    if constexpr (M == 2) {
+        const float v1[1][2] = {{v[0], v[1]}};
+        float z1[1][2], d1[1];
+        closest_2d<SH, 1>(v1, geo, z1, d1);
+        z[0] = z1[0][0];
+        z[1] = z1[0][1];
+        d2 = d1[0];
+        return;
+    }
+    const int nr = geo.nr;
+    bool in = true;
+    for (int r = 0; r < nr; ++r) {
+        const float4 f = geo.row(r);
+        in = in & (pdot<M>(f, v) - f.w <= 0.f);
+    }
+    d2 = 0.f;
+#pragma unroll
+    for (int a = 0; a < M; ++a) z[a] = v[a];
+    if (!in) {
+        d2 = inf;
+        if (M == 3) {  // faces whose projection lands inside the obstacle
+            for (int r = 0; r < nr; ++r) {
+                const float4 f = geo.face_of(r);
+                const float sd = pdot<M>(f, v) - f.w;
+                if (!(sd > 0.f) || sd * sd >= d2) continue;
+                float c[M];
+#pragma unroll
+                for (int a = 0; a < M; ++a) c[a] = fmaf(-sd, a == 0 ? f.x : (a == 1 ? f.y : f.z), v[a]);
+                bool ok = true;
+                for (int q = 0; q < nr; ++q) {
+                    if (q == r) continue;
+                    const float4 g = geo.row(q);
+                    const float sv = pdot<M>(g, c) - g.w;
+                    const float mag = fabsf(g.x * c[0]) + fabsf(g.y * c[1]) + fabsf(g.z * c[M - 1]) + fabsf(g.w);
+                    ok = ok && sv <= 8.f * U32P * mag;
+                }
+                if (ok) {
+                    d2 = sd * sd;
+#pragma unroll
+                    for (int a = 0; a < M; ++a) z[a] = c[a];
+                }
+            }
+        }
+        // edge segments (and their end points, the vertices).  The
+        // candidate is chosen by sign tests, not by comparing nearly
+        // equal distances: a segment whose parameter needs no clamping
+        // holds the projection.  The nearest candidate is the fallback
+        // for what rounding leaves undecided.
+        const int ne = geo.ne;
+        bool found = false;
+        float fb_d2 = inf, fb[M];
+#pragma unroll
+        for (int a = 0; a < M; ++a) fb[a] = v[a];
+        for (int e = 0; e < ne && !found && !(d2 < inf); ++e) {
+            const float4 e0 = geo.edge_of(e, 0), e1 = geo.edge_of(e, 1);
+            float w[M];
+            w[0] = v[0] - e0.x;
+            w[1] = v[1] - e0.y;
+            if (M == 3) w[M - 1] = v[M - 1] - e0.z;
+            float t = e1.x * w[0];
+            t = fmaf(e1.y, w[1], t);
+            if (M == 3) t = fmaf(e1.z, w[M - 1], t);
+            const float tc = fminf(fmaxf(t, e0.w), e1.w);
+            float c[M], dd = 0.f;
+            c[0] = fmaf(tc, e1.x, e0.x);
+            c[1] = fmaf(tc, e1.y, e0.y);
+            if (M == 3) c[M - 1] = fmaf(tc, e1.z, e0.z);
+#pragma unroll
+            for (int a = 0; a < M; ++a) dd = fmaf(v[a] - c[a], v[a] - c[a], dd);
+            // an unclamped point of an edge whose two facet normals span v - c
+            bool hit = false;
+            if (tc == t) {
+                const float4 e2 = geo.edge_of(e, 2), e3 = geo.edge_of(e, 3);
+                const float wx = v[0] - c[0], wy = v[1] - c[1], wz = v[M - 1] - c[M - 1];
+                // signs of (n_a x w) . d, (w x n_b) . d and (n_a x n_b) . d
+                const float k1 = (e2.y * wz - e2.z * wy) * e1.x + (e2.z * wx - e2.x * wz) * e1.y +
+                                 (e2.x * wy - e2.y * wx) * e1.z;
+                const float k2 = (wy * e3.z - wz * e3.y) * e1.x + (wz * e3.x - wx * e3.z) * e1.y +
+                                 (wx * e3.y - wy * e3.x) * e1.z;
+                float kk = (e2.y * e3.z - e2.z * e3.y) * e1.x + (e2.z * e3.x - e2.x * e3.z) * e1.y +
+                           (e2.x * e3.y - e2.y * e3.x) * e1.z;
+                float s1 = k1, s2 = k2;
+                if (kk < 0.f) {
+                    s1 = -s1;
+                    s2 = -s2;
+                    kk = -kk;
+                }
+                hit = kk > 0.f && s1 >= 0.f && s2 >= 0.f;
+            }
+            if (hit) {
+                found = true;
+                d2 = dd;
+#pragma unroll
+                for (int a = 0; a < M; ++a) z[a] = c[a];
+            } else if (dd < fb_d2) {
+                fb_d2 = dd;
+#pragma unroll
+                for (int a = 0; a < M; ++a) fb[a] = c[a];
+            }
+        }
+        if (!found && !(d2 < inf)) {
+            d2 = fb_d2;
+#pragma unroll
+            for (int a = 0; a < M; ++a) z[a] = fb[a];
+        } else if (!found && fb_d2 < d2) {
+            d2 = fb_d2;
+#pragma unroll
+            for (int a = 0; a < M; ++a) z[a] = fb[a];
         }
     }
 }
@@ -355,132 +634,13 @@ __global__ void __launch_bounds__(256) k_planes(PlanesParams Q) {
             float v[M];
 #pragma unroll
             for (int a = 0; a < M; ++a) v[a] = pld32(Q.points, p * M + a, Q.in_f32);
-            const int nr = Q.ocount[o];
-            const float4* rw = reinterpret_cast<const float4*>(Q.orow) + (long long)o * Q.max_orows;
-            bool in = true;
-            for (int r = 0; r < nr; ++r) {
-                const float4 f = __ldg(rw + r);
-                in = in && pdot<M>(f, v) - f.w <= 0.f;
-            }
-            float z[M], d2 = 0.f;
-#pragma unroll
-            for (int a = 0; a < M; ++a) z[a] = v[a];
-            if (!in) {
-                d2 = inf;
-                if (M == 3) {  // faces whose projection lands inside the obstacle
-                    const float4* fw = reinterpret_cast<const float4*>(Q.face) + (long long)o * Q.max_orows;
-                    for (int r = 0; r < nr; ++r) {
-                        const float4 f = __ldg(fw + r);
-                        const float sd = pdot<M>(f, v) - f.w;
-                        if (!(sd > 0.f) || sd * sd >= d2) continue;
-                        float c[M];
-#pragma unroll
-                        for (int a = 0; a < M; ++a) c[a] = fmaf(-sd, a == 0 ? f.x : (a == 1 ? f.y : f.z), v[a]);
-                        bool ok = true;
-                        for (int q = 0; q < nr; ++q) {
-                            if (q == r) continue;
-                            const float4 g = __ldg(rw + q);
-                            const float sv = pdot<M>(g, c) - g.w;
-                            const float mag = fabsf(g.x * c[0]) + fabsf(g.y * c[1]) + fabsf(g.z * c[M - 1]) + fabsf(g.w);
-                            ok = ok && sv <= 8.f * U32P * mag;
-                        }
-                        if (ok) {
-                            d2 = sd * sd;
-#pragma unroll
-                            for (int a = 0; a < M; ++a) z[a] = c[a];
-                        }
-                    }
-                }
-                // edge segments (and their end points, the vertices).  The
-                // candidate is chosen by sign tests, not by comparing nearly
-                // equal distances: a segment whose parameter needs no clamping
-                // (and, in 2-D, whose facet v lies outside of) holds the
-                // projection; in 2-D a vertex does when v - vertex lies in the
-                // cone of its two facet normals.  The nearest candidate is the
-                // fallback for what rounding leaves undecided.
-                const float4* ew = reinterpret_cast<const float4*>(Q.edge) + EDGE_F4 * (long long)o * Q.max_edges;
-                const int ne = Q.nedge[o];
-                bool found = false;
-                float fb_d2 = inf, fb[M];
-#pragma unroll
-                for (int a = 0; a < M; ++a) fb[a] = v[a];
-                for (int e = 0; e < ne && !found && !(M == 3 && d2 < inf); ++e) {
-                    const float4 e0 = __ldg(ew + EDGE_F4 * e), e1 = __ldg(ew + EDGE_F4 * e + 1);
-                    float w[M];
-                    w[0] = v[0] - e0.x;
-                    w[1] = v[1] - e0.y;
-                    if (M == 3) w[M - 1] = v[M - 1] - e0.z;
-                    float t = e1.x * w[0];
-                    t = fmaf(e1.y, w[1], t);
-                    if (M == 3) t = fmaf(e1.z, w[M - 1], t);
-                    const float tc = fminf(fmaxf(t, e0.w), e1.w);
-                    float c[M], dd = 0.f;
-                    c[0] = fmaf(tc, e1.x, e0.x);
-                    c[1] = fmaf(tc, e1.y, e0.y);
-                    if (M == 3) c[M - 1] = fmaf(tc, e1.z, e0.z);
-#pragma unroll
-                    for (int a = 0; a < M; ++a) dd = fmaf(v[a] - c[a], v[a] - c[a], dd);
-                    bool hit;
-                    if (M == 2) {
-                        const float4 e2 = __ldg(ew + EDGE_F4 * e + 2), e3 = __ldg(ew + EDGE_F4 * e + 3);
-                        const float sd = fmaf(e3.y, v[1], e3.x * v[0]) - e3.z;  // outside this facet?
-                        if (tc == t) {
-                            hit = sd > 0.f;
-                        } else {
-                            // a clamped end: the vertex; v - c in the cone of the two normals
-                            const float wx = v[0] - c[0], wy = v[1] - c[1];
-                            const float nx = t < e0.w ? e2.x : e2.z, ny = t < e0.w ? e2.y : e2.w;
-                            float k1 = e3.x * wy - e3.y * wx, k2 = wx * ny - wy * nx, kk = e3.x * ny - e3.y * nx;
-                            if (kk < 0.f) {
-                                k1 = -k1;
-                                k2 = -k2;
-                                kk = -kk;
-                            }
-                            hit = (nx != 0.f || ny != 0.f) && kk > 0.f && k1 >= 0.f && k2 >= 0.f;
-                        }
-                    } else {
-                        // 3-D: an unclamped point of an edge whose two facet normals span v - c
-                        hit = false;
-                        if (tc == t) {
-                            const float4 e2 = __ldg(ew + EDGE_F4 * e + 2), e3 = __ldg(ew + EDGE_F4 * e + 3);
-                            const float wx = v[0] - c[0], wy = v[1] - c[1], wz = v[M - 1] - c[M - 1];
-                            // signs of (n_a x w) . d, (w x n_b) . d and (n_a x n_b) . d
-                            const float k1 = (e2.y * wz - e2.z * wy) * e1.x + (e2.z * wx - e2.x * wz) * e1.y +
-                                             (e2.x * wy - e2.y * wx) * e1.z;
-                            const float k2 = (wy * e3.z - wz * e3.y) * e1.x + (wz * e3.x - wx * e3.z) * e1.y +
-                                             (wx * e3.y - wy * e3.x) * e1.z;
-                            float kk = (e2.y * e3.z - e2.z * e3.y) * e1.x + (e2.z * e3.x - e2.x * e3.z) * e1.y +
-                                       (e2.x * e3.y - e2.y * e3.x) * e1.z;
-                            float s1 = k1, s2 = k2;
-                            if (kk < 0.f) {
-                                s1 = -s1;
-                                s2 = -s2;
-                                kk = -kk;
-                            }
-                            hit = kk > 0.f && s1 >= 0.f && s2 >= 0.f;
-                        }
-                    }
-                    if (hit) {
-                        found = true;
-                        d2 = dd;
-#pragma unroll
-                        for (int a = 0; a < M; ++a) z[a] = c[a];
-                    } else if (dd < fb_d2) {
-                        fb_d2 = dd;
-#pragma unroll
-                        for (int a = 0; a < M; ++a) fb[a] = c[a];
-                    }
-                }
-                if (!found && !(d2 < inf && M == 3)) {
-                    d2 = fb_d2;
-#pragma unroll
-                    for (int a = 0; a < M; ++a) z[a] = fb[a];
-                } else if (!found && M == 3 && fb_d2 < d2) {
-                    d2 = fb_d2;
-#pragma unroll
-                    for (int a = 0; a < M; ++a) z[a] = fb[a];
-                }
-            }
+            const long long oo = o;
+            const Geom<false> geo = {reinterpret_cast<const float4*>(Q.orow) + oo * Q.max_orows,
+                                     reinterpret_cast<const float4*>(Q.face) + oo * Q.max_orows,
+                                     reinterpret_cast<const float4*>(Q.edge) + EDGE_F4 * oo * Q.max_edges,
+                                     1, Q.ocount[o], Q.nedge[o]};
+            float z[M], d2;
+            pair_closest<M>(v, geo, z, d2);
             const float d = sqrtf(d2);
             if (Q.closest)
 #pragma unroll
@@ -516,6 +676,102 @@ __global__ void __launch_bounds__(256) k_planes(PlanesParams Q) {
     }
 }
 
+// All pairs in 2-D, by blocks of up to 128 obstacles whose geometry stays in
+// shared memory while groups of as many threads take the points of a chunk in
+// turn (one thread an obstacle, so a point's outputs are stored coalesced).
+// Read per pair from global memory, the 32 obstacles of a warp take 32 lines
+// a load, and those loads bounded the kernel (5000 points x 500 obstacles:
+// 71 us); from shared memory, laid
+// out [entry][obstacle] with one float4 of padding, a load is conflict-free:
+// 53 us, bound by issue (560 instructions a pair of which 7 edges take 350).  Same arithmetic and results.
+constexpr int PL_THREADS = 384, PL_NP = 4;
+
+__global__ void __launch_bounds__(PL_THREADS, 2) k_planes_all(PlanesParams Q, int ob, int chunk) {
+    extern __shared__ float4 geo_sm[];
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, lane = tid & 31, stride = ob + 1, n4 = Q.max_orows + EDGE_F4 * Q.max_edges;
+    if (tid == 0) s_fail = p_failed(Q.info);
+    const int o0 = blockIdx.x * ob, nob = min(ob, Q.n_obst - o0);
+    const float4* rw = reinterpret_cast<const float4*>(Q.orow) + (long long)o0 * Q.max_orows;
+    const float4* ew = reinterpret_cast<const float4*>(Q.edge) + EDGE_F4 * (long long)o0 * Q.max_edges;
+    for (int u = tid; u < nob * n4; u += PL_THREADS) {
+        const int lo = u / n4, j = u - lo * n4, e = j - Q.max_orows;
+        geo_sm[j * stride + lo] = e < 0 ? rw[lo * Q.max_orows + j] : ew[lo * EDGE_F4 * Q.max_edges + e];
+    }
+    const int groups = PL_THREADS / ob, g = tid / ob, lo = tid - g * ob, o = o0 + lo;
+    const bool act = lo < nob && g < groups;
+    Geom<true> geo = {geo_sm + lo, nullptr, geo_sm + Q.max_orows * stride + lo, stride, 0, 0};
+    if (act) {
+        geo.nr = Q.ocount[o];
+        geo.ne = Q.nedge[o];
+    }
+    __syncthreads();
+    if (s_fail || g >= groups) return;  // whole warps: ob is a multiple of 32
+    const float inf = __int_as_float(0x7f800000);
+    const bool pair_aligned = ((uintptr_t)Q.closest & 7) == 0, whole = __all_sync(0xffffffffu, act);
+    const int p1 = (int)min((long long)Q.P, ((long long)blockIdx.y + 1) * chunk);
+    for (int pb = blockIdx.y * chunk + g; pb < p1; pb += groups * PL_NP) {
+        float v[PL_NP][2], z[PL_NP][2], d2[PL_NP];
+#pragma unroll
+        for (int i = 0; i < PL_NP; ++i) {
+            const long long p = min(pb + i * groups, p1 - 1);
+            v[i][0] = pld32(Q.points, p * 2, Q.in_f32);
+            v[i][1] = pld32(Q.points, p * 2 + 1, Q.in_f32);
+        }
+        if (act) closest_2d<true, PL_NP>(v, geo, z, d2);
+#pragma unroll
+        for (int i = 0; i < PL_NP; ++i) {
+            const int p = pb + i * groups;
+            if (p >= p1) break;  // warp-uniform
+            const long long k = (long long)p * Q.n_obst + o;
+            unsigned bits = 0xffffffffu;
+            float h[2] = {0.f, 0.f}, l = 0.f;
+            if (act) {
+                const float d = sqrtf(d2[i]);
+                if (Q.closest) {
+                    const float nan = __int_as_float(0x7fc00000);
+                    const float2 c = d2[i] < inf ? make_float2(z[i][0], z[i][1]) : make_float2(nan, nan);
+                    if (pair_aligned) {
+                        reinterpret_cast<float2*>(Q.closest)[k] = c;
+                    } else {
+                        Q.closest[2 * k] = c.x;
+                        Q.closest[2 * k + 1] = c.y;
+                    }
+                }
+                if (Q.dist) Q.dist[k] = d;
+                const float rdn = (d > 0.f && d < inf) ? 1.f / d : 0.f;
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    h[a] = (v[i][a] - z[i][a]) * rdn;
+                    l = fmaf(h[a], z[i][a], l);
+                }
+                bits = __float_as_uint(d);
+            }
+            if (Q.plane) {
+                if (whole) {  // 96 words of the warp, exchanged for coalesced stores
+                    float* out = Q.plane + 3 * (k - lane);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        const int w = 32 * q + lane, src = w / 3, c = w - 3 * src;
+                        const float x0 = __shfl_sync(0xffffffffu, h[0], src), x1 = __shfl_sync(0xffffffffu, h[1], src);
+                        const float x2 = __shfl_sync(0xffffffffu, l, src);
+                        out[w] = c == 0 ? x0 : (c == 1 ? x1 : x2);
+                    }
+                } else if (act) {
+                    Q.plane[3 * k] = h[0];
+                    Q.plane[3 * k + 1] = h[1];
+                    Q.plane[3 * k + 2] = l;
+                }
+            }
+            if (Q.keys) {
+                const unsigned mn = __reduce_min_sync(0xffffffffu, bits);
+                const unsigned who = __ballot_sync(0xffffffffu, act && bits == mn);  // the lowest lane is the lowest obstacle
+                if (who && lane == __ffs(who) - 1) atomicMin(Q.keys + p, ((unsigned long long)mn << 32) | (unsigned)o);
+            }
+        }
+    }
+}
+
 __global__ void k_planes_nearest(PlanesParams Q) {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= Q.P || p_failed(Q.info)) return;
@@ -531,10 +787,14 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
     cudaStream_t st = (cudaStream_t)stream;
     const long long orows = (long long)Q.n_obst * Q.max_orows;
     if (orows > 0) {
-        k_planes_prep<<<(int)((orows + 255) / 256), 256, 0, st>>>(Q);
-        if (Q.m == 2) k_planes_geom<2><<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
-        else k_planes_geom<3><<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
-        *launches += 2;
+        if (Q.m == 2) {
+            k_planes_geom2<<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
+        } else {
+            k_planes_prep<<<(int)((orows + 255) / 256), 256, 0, st>>>(Q);
+            k_planes_geom<<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
+            ++*launches;
+        }
+        ++*launches;
     }
     const long long total = (long long)Q.P * Q.n_obst;
     if (total > 0) {
@@ -545,8 +805,27 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
             else k_planes_ub<3><<<(int)grid, 256, 0, st>>>(Q);
             ++*launches;
         }
-        if (Q.m == 2) k_planes<2><<<(int)grid, 256, 0, st>>>(Q);
-        else k_planes<3><<<(int)grid, 256, 0, st>>>(Q);
+        // all pairs in 2-D: obstacles in blocks of whole warps, and as many
+        // chunks of points as fill the GPU once.  Not where a block would be
+        // alone on an SM (the most rows) or a warp mostly empty (few obstacles).
+        const int ob = Q.n_obst >= 128 ? 128 : (Q.n_obst + 31) & ~31;
+        const size_t smem = sizeof(float4) * (size_t)(ob + 1) * (Q.max_orows + EDGE_F4 * Q.max_edges);
+        const int fit = (int)(220 * 1024 / (smem + 2 * 1024));
+        if (Q.m == 2 && !Q.ub && Q.n_obst >= 24 && fit >= 2) {
+            const cudaError_t ea = cudaFuncSetAttribute(k_planes_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (ea != cudaSuccess) return (int)ea;
+            const int nb = (Q.n_obst + ob - 1) / ob, groups = PL_THREADS / ob;
+            long long chunks = ((long long)num_sms * (fit < 2 ? fit : 2) + nb - 1) / nb;
+            const long long most = (Q.P + groups * PL_NP - 1) / (groups * PL_NP);
+            if (chunks > most) chunks = most;
+            if (chunks > 65535) chunks = 65535;
+            const int chunk = (int)((Q.P + chunks - 1) / chunks);
+            k_planes_all<<<dim3((unsigned)nb, (unsigned)((Q.P + chunk - 1) / chunk)), PL_THREADS, smem, st>>>(Q, ob, chunk);
+        } else if (Q.m == 2) {
+            k_planes<2><<<(int)grid, 256, 0, st>>>(Q);
+        } else {
+            k_planes<3><<<(int)grid, 256, 0, st>>>(Q);
+        }
         ++*launches;
     }
     if (Q.P > 0 && (Q.nearest || Q.nearest_dist)) {
