@@ -1,6 +1,7 @@
-// Differentiable refinement objective for sm_103a: one thread per Bezier
-// segment (the axes one after the other), forward (loss) and hand-written backward (d loss / d control points
-// and d loss / d T) of
+// Differentiable refinement objective for sm_103a: M threads per Bezier
+// segment (one an axis of the reach margins and the snap energy, and two of
+// the interior control points of the free margins), forward (loss) and
+// hand-written backward (d loss / d control points and d loss / d T) of
 //
 //   loss = w_snap J_snap + mu sum_r phi_delta(margin_r)
 //
@@ -26,184 +27,270 @@ namespace plan {
 
 namespace {
 
-DEVI float phi_f(float m, float delta, float log_delta) {
-    if (m >= delta) return -logf(m);
-    const float z = (m - 2.f * delta) / delta;
-    return -log_delta + 0.5f * z * z - 0.5f;
+// The relaxed barrier's constants: value and slope of the quadratic below delta.
+struct Barrier {
+    float delta, inv, inv2, off;  // delta, 1 / delta, 1 / delta^2, -log delta - 1/2
+};
+
+// phi(m) and, with GRAD, phi'(m) of one margin.
+template <bool GRAD>
+DEVI float phi_one(const Barrier& B, float m, float& slope) {
+    const bool in = m >= B.delta;
+    const float z = (m - 2.f * B.delta) * B.inv;
+    if (GRAD) slope = in ? -1.f / m : (m - 2.f * B.delta) * B.inv2;
+    return in ? -logf(m) : fmaf(0.5f * z, z, B.off);
 }
-DEVI float dphi_f(float m, float delta) { return m >= delta ? -1.f / m : (m - 2.f * delta) / (delta * delta); }
 
-constexpr float fact_f(int n) { return n <= 1 ? 1.f : n * fact_f(n - 1); }
-constexpr int comb_i(int n, int k) { return (k < 0 || k > n) ? 0 : (k == 0 || k == n ? 1 : comb_i(n - 1, k - 1) + comb_i(n - 1, k)); }
+// phi(c - Q) + phi(c + Q) and its derivative in Q.  Both margins in the
+// logarithm share one root of work: log m1 + log m2 = log(m1 m2), and the two
+// reciprocals come from one (m1 + m2 = 2 c, so the product stays in range for
+// every bound below 2^60; a larger one takes the margins one by one).
+template <bool GRAD>
+DEVI float phi_pair(const Barrier& B, float c, float Q, float& slope) {
+    const float m1 = c - Q, m2 = c + Q;
+    if (c > 1.152921504606847e18f) {
+        float s1 = 0.f, s2 = 0.f;
+        const float v = phi_one<GRAD>(B, m1, s1) + phi_one<GRAD>(B, m2, s2);
+        if (GRAD) slope = s2 - s1;
+        return v;
+    }
+    const bool in1 = m1 >= B.delta, in2 = m2 >= B.delta;
+    const float u1 = in1 ? m1 : 1.f, u2 = in2 ? m2 : 1.f, pr = u1 * u2;
+    const float d1 = m1 - 2.f * B.delta, d2 = m2 - 2.f * B.delta;
+    const float z1 = d1 * B.inv, z2 = d2 * B.inv;
+    float v = -logf(pr);
+    v += in1 ? 0.f : fmaf(0.5f * z1, z1, B.off);
+    v += in2 ? 0.f : fmaf(0.5f * z2, z2, B.off);
+    if (GRAD) {
+        const float r = 1.f / pr;
+        const float s1 = in1 ? -r * u2 : d1 * B.inv2, s2 = in2 ? -r * u1 : d2 * B.inv2;
+        slope = s2 - s1;
+    }
+    return v;
+}
 
-template <int M, int L>
-DEVI void fwd_diff(float (&d)[8][M], int len) {  // d[0..len-2] = d[j+1] - d[j]
+// Constants of degree PD, formed at compile time: kept as an object, because a
+// constexpr function called in an unrolled loop is compiled as a call.
+template <int PD>
+struct RefineConst {
+    float scale[5];               // p! / (p-k)!, k = 0 .. 4
+    float gram[PD - 3][PD - 3];   // C(q,j) C(q,l) / ((2q+1) C(2q,j+l)), q = PD - 4
+};
+template <int PD>
+constexpr RefineConst<PD> refine_const() {
+    RefineConst<PD> c{};
+    c.scale[0] = 1.f;
+    for (int k = 1; k <= 4; ++k) c.scale[k] = c.scale[k - 1] * (float)(PD - k + 1);
+    constexpr int q = PD - 4;
+    long long C[2 * q + 1][2 * q + 1] = {};
+    for (int n = 0; n <= 2 * q; ++n)
+        for (int k = 0; k <= n; ++k) C[n][k] = (k == 0 || k == n) ? 1 : C[n - 1][k - 1] + C[n - 1][k];
+    for (int j = 0; j <= q; ++j)
+        for (int l = 0; l <= q; ++l) c.gram[j][l] = (float)(C[q][j] * C[q][l]) / (float)((2 * q + 1) * C[2 * q][j + l]);
+    return c;
+}
+
+template <int L>
+DEVI void fwd_diff(float (&d)[L], int len) {  // d[0..len-2] = d[j+1] - d[j]
 #pragma unroll
     for (int j = 0; j < L - 1; ++j)
-        if (j < len - 1)
-#pragma unroll
-            for (int a = 0; a < M; ++a) d[j][a] = d[j + 1][a] - d[j][a];
+        if (j < len - 1) d[j] = d[j + 1] - d[j];
 }
 
 // adjoint of the forward difference: g has `len` entries -> len+1 entries
-template <int M, int L>
-DEVI void adj_diff(float (&g)[8][M], int len) {
-    float out[8][M];
+template <int L>
+DEVI void adj_diff(float (&g)[L], int len) {
+    float prev = 0.f;
 #pragma unroll
     for (int l = 0; l < L; ++l)
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            float v = 0.f;
-            if (l >= 1 && l - 1 < len) v += g[l - 1][a];
-            if (l < len) v -= g[l][a];
-            out[l][a] = (l <= len) ? v : 0.f;
+        if (l <= len) {
+            const float cur = l < len ? g[l] : 0.f;
+            g[l] = prev - cur;
+            prev = cur;
         }
-#pragma unroll
-    for (int l = 0; l < L; ++l)
-#pragma unroll
-        for (int a = 0; a < M; ++a) g[l][a] = out[l][a];
 }
 
 }  // namespace
 
-template <int M, int G, int PD, bool GRAD>
-__global__ void __launch_bounds__(128) k_refine(RefineParams R) {
-    constexpr int L = PD + 1;
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (s >= R.S) return;
-    const float* Ps = R.P + s * L * M;
-    const float T = R.T[s];
-    const float Ti = 1.f / T;
-    const float mu = R.mu, delta = R.delta, ld = logf(R.delta), ws = R.w_snap;
-    const float up = GRAD ? R.grad_loss[s] : 1.f;
-    float loss = 0.f, dT = 0.f;
-    float* dPs = GRAD ? R.dP + s * L * M : nullptr;
+// A CTA takes RF_SEGS consecutive segments: their control points, rows and
+// bounds come in coalesced (each a contiguous run of the input), and the
+// gradients go out the same way, all through shared memory (per-segment
+// strides odd, so that threads of different segments hit different banks).
+//
+// One thread a segment took 59 us forward and 80 us backward for 65,536 3-D
+// segments: 2048 warps waited for strided loads, and the snap energy's
+// binomials were formed by recursive calls at run time (a third of all
+// instructions and most of the memory traffic, to the call stack).  M threads a
+// segment balance (18 reach rows and 2 of 6 interior points' rows each), have no
+// global load inside the loops and share one logarithm and one reciprocal
+// between the two margins of a reach row: 21 and 30 us, bound by issue.
+constexpr int RF_SEGS = 64;
+constexpr int RF_ROWS = 16;  // polytope rows staged at a time
 
-    // Reach margins and snap energy separate over the axes (Theorem 1 per
-    // axis; the snap integral is the sum of the axes' integrals): one axis
-    // at a time keeps few values live.  Its gradient goes straight to dP.
-#pragma unroll 1
-    for (int a = 0; a < M; ++a) {
-        float Pa[8][1];
+template <int M, int G, int PD, bool GRAD>
+__global__ void __launch_bounds__(RF_SEGS * M) k_refine(RefineParams R) {
+    constexpr int L = PD + 1, NT = RF_SEGS * M, PS = (L * M) | 1, AS = (RF_ROWS * M) | 1, BS = RF_ROWS | 1;
+    static_assert(PD - 1 == 2 * M, "two interior control points a thread");
+    constexpr RefineConst<PD> K = refine_const<PD>();
+    __shared__ float sP[RF_SEGS * PS];                // [segment][PS] control points
+    __shared__ float sG[GRAD ? RF_SEGS * PS : 1];     // their gradient
+    __shared__ float sA[RF_SEGS * AS], sB[RF_SEGS * BS];  // [segment][rows of a chunk]
+    __shared__ float s_red[2][NT];                    // loss and dT parts
+    const int tid = threadIdx.x, rmax = R.rmax;
+    const long long s0 = (long long)blockIdx.x * RF_SEGS;
+    const int ns = (int)min((long long)RF_SEGS, R.S - s0);
+    auto stage_rows = [&](int c0) {  // rows c0 .. c0 + RF_ROWS of every segment
+        const int rc = min(RF_ROWS, rmax - c0);
+        for (int u = tid; u < ns * rc * M; u += NT) {
+            const int sg = u / (rc * M), x = u - sg * rc * M;
+            sA[sg * AS + x] = R.A[((s0 + sg) * rmax + c0) * M + x];
+        }
+        for (int u = tid; u < ns * rc; u += NT) {
+            const int sg = u / rc, x = u - sg * rc;
+            sB[sg * BS + x] = R.b[(s0 + sg) * rmax + c0 + x];
+        }
+    };
+    for (int u = tid; u < ns * L * M; u += NT) sP[u / (L * M) * PS + u % (L * M)] = R.P[s0 * L * M + u];
+    if (rmax > 0) stage_rows(0);
+    const int q = tid / M, a = tid - q * M;  // segment of the block, axis
+    const bool act = q < ns;
+    const float T = act ? R.T[s0 + q] : 1.f, up = GRAD && act ? R.grad_loss[s0 + q] : 1.f;
+    const int nr = act ? min(R.nrows[s0 + q], rmax) : 0;
+    __syncthreads();
+    const float mu = R.mu, ws = R.w_snap, Ti = 1.f / T;
+    const Barrier B = {R.delta, 1.f / R.delta, 1.f / (R.delta * R.delta), -logf(R.delta) - 0.5f};
+    float loss = 0.f, dT = 0.f;
+    if (act) {
+        // reach margins and snap energy of axis a (Theorem 1 per axis; the snap
+        // integral is the sum of the axes' integrals)
+        float Pa[L], ga[L];
 #pragma unroll
-        for (int l = 0; l < 8; ++l) Pa[l][0] = l < L ? Ps[l * M + a] : 0.f;
-        float ga[8];
+        for (int l = 0; l < L; ++l) {
+            Pa[l] = sP[q * PS + l * M + a];
+            ga[l] = 0.f;
+        }
+        float d[L], pk = 1.f;
 #pragma unroll
-        for (int l = 0; l < 8; ++l) ga[l] = 0.f;
+        for (int l = 0; l < L; ++l) d[l] = Pa[l];
 #pragma unroll
         for (int k = 1; k <= G; ++k) {
-            float d[8][1];
+            fwd_diff<L>(d, L - k + 1);  // the k-th differences
+            pk *= Ti;
+            const float sk = K.scale[k] * pk, ck = R.bound[k - 1];
+            float g[L], dk = 0.f;
 #pragma unroll
-            for (int l = 0; l < 8; ++l) d[l][0] = Pa[l][0];
-#pragma unroll
-            for (int it = 0; it < k; ++it) fwd_diff<1, L>(d, L - it);
-            float sk = fact_f(PD) / fact_f(PD - k);
-#pragma unroll
-            for (int it = 0; it < k; ++it) sk *= Ti;
-            const float ck = R.bound[k - 1];
-            const int nk = L - k;
-            float g[8][1];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                g[j][0] = 0.f;
-                if (j < nk) {
-                    const float Q = sk * d[j][0];
-                    const float m1 = ck - Q, m2 = ck + Q;
-                    loss += mu * (phi_f(m1, delta, ld) + phi_f(m2, delta, ld));
+            for (int j = 0; j < L; ++j) {
+                g[j] = 0.f;
+                if (j < L - k) {
+                    const float Q = sk * d[j];
+                    float sl = 0.f;
+                    loss += phi_pair<GRAD>(B, ck, Q, sl);
                     if (GRAD) {
-                        const float gQ = mu * (dphi_f(m2, delta) - dphi_f(m1, delta)) * up;
-                        g[j][0] = gQ * sk;
-                        dT += gQ * Q * (-(float)k) * Ti;
+                        g[j] = sl * sk;
+                        dk = fmaf(sl, Q, dk);
                     }
                 }
             }
             if (GRAD) {
+                dT = fmaf(-(float)k, dk, dT);
 #pragma unroll
-                for (int it = k; it >= 1; --it) adj_diff<1, L>(g, L - it);
+                for (int it = k; it >= 1; --it) adj_diff<L>(g, L - it);
 #pragma unroll
-                for (int l = 0; l < L; ++l) ga[l] += g[l][0];
+                for (int l = 0; l < L; ++l) ga[l] += g[l];
             }
         }
+        loss *= mu;
+        dT *= mu * Ti;
         {
-            constexpr int q = PD - 4;
-            float d4[8][1];
+            constexpr int qd = PD - 4;
 #pragma unroll
-            for (int l = 0; l < 8; ++l) d4[l][0] = Pa[l][0];
-#pragma unroll
-            for (int it = 0; it < 4; ++it) fwd_diff<1, L>(d4, L - it);
-            float c = fact_f(PD) / fact_f(PD - 4);
-            c = c * c;
+            for (int it = G; it < 4; ++it) fwd_diff<L>(d, L - it);
+            float c = K.scale[4] * K.scale[4];
             float t7 = Ti * Ti * Ti;
             t7 = t7 * t7 * Ti;
             c *= t7;
-            float quad = 0.f;
-            float gd[8][1];
+            float quad = 0.f, gd[L];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) gd[j][0] = 0.f;
+            for (int j = 0; j < L; ++j) gd[j] = 0.f;
 #pragma unroll
-            for (int j = 0; j <= q; ++j)
+            for (int j = 0; j <= qd; ++j)
 #pragma unroll
-                for (int l = 0; l <= q; ++l) {
-                    const float Gjl = (float)(comb_i(q, j) * comb_i(q, l)) / (float)((2 * q + 1) * comb_i(2 * q, j + l));
-                    quad = fmaf(Gjl * d4[j][0], d4[l][0], quad);
-                    if (GRAD) gd[j][0] = fmaf(Gjl, d4[l][0], gd[j][0]);
+                for (int l = 0; l <= qd; ++l) {
+                    const float Gjl = K.gram[j][l];
+                    quad = fmaf(Gjl * d[j], d[l], quad);
+                    if (GRAD) gd[j] = fmaf(Gjl, d[l], gd[j]);
                 }
             const float J = c * quad;
             loss += ws * J;
             if (GRAD) {
-                const float f = ws * c * 2.f * up;
+                const float f = ws * c * 2.f;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) gd[j][0] = (j <= q) ? gd[j][0] * f : 0.f;
+                for (int it = 4; it >= 1; --it) adj_diff<L>(gd, L - it);
 #pragma unroll
-                for (int it = 4; it >= 1; --it) adj_diff<1, L>(gd, L - it);
-#pragma unroll
-                for (int l = 0; l < L; ++l) ga[l] += gd[l][0];
-                dT += ws * (-7.f) * J * Ti * up;
-            }
-        }
-        if (GRAD) {
-#pragma unroll
-            for (int l = 0; l < L; ++l) dPs[l * M + a] = ga[l];
-        }
-    }
-    // free-space margins of the interior control points (every axis)
-    float P[8][M];
-#pragma unroll
-    for (int l = 1; l < PD; ++l)
-#pragma unroll
-        for (int a = 0; a < M; ++a) P[l][a] = Ps[l * M + a];
-    float df[8][M];
-#pragma unroll
-    for (int l = 0; l < 8; ++l)
-#pragma unroll
-        for (int a = 0; a < M; ++a) df[l][a] = 0.f;
-    const int nr = min(R.nrows[s], R.rmax);
-    for (int r = 0; r < nr; ++r) {
-        float Ar[M];
-#pragma unroll
-        for (int a = 0; a < M; ++a) Ar[a] = R.A[(s * R.rmax + r) * M + a];
-        const float br = R.b[s * R.rmax + r];
-#pragma unroll
-        for (int l = 1; l < PD; ++l) {
-            float dot = 0.f;
-#pragma unroll
-            for (int a = 0; a < M; ++a) dot = fmaf(Ar[a], P[l][a], dot);
-            const float mg = br - dot;
-            loss += mu * phi_f(mg, delta, ld);
-            if (GRAD) {
-                const float gm = mu * dphi_f(mg, delta) * up;
-#pragma unroll
-                for (int a = 0; a < M; ++a) df[l][a] -= gm * Ar[a];
+                for (int l = 0; l < L; ++l) sG[q * PS + l * M + a] = fmaf(f, gd[l], mu * ga[l]) * up;
+                dT += ws * (-7.f) * J * Ti;
             }
         }
     }
-    if (R.loss) R.loss[s] = loss;
+    // free margins of control points 2a+1 and 2a+2
+    float fl = 0.f, P2[2][M], df[2][M];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < M; ++c) {
+            P2[i][c] = act ? sP[q * PS + (2 * a + 1 + i) * M + c] : 0.f;
+            df[i][c] = 0.f;
+        }
+    for (int c0 = 0; c0 < rmax; c0 += RF_ROWS) {
+        if (c0 > 0) {
+            __syncthreads();
+            stage_rows(c0);
+            __syncthreads();
+        }
+        const int n = min(nr - c0, RF_ROWS);
+        for (int r = 0; r < n; ++r) {
+            float Ar[M];
+#pragma unroll
+            for (int c = 0; c < M; ++c) Ar[c] = sA[q * AS + r * M + c];
+            const float br = sB[q * BS + r];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float dot = 0.f;
+#pragma unroll
+                for (int c = 0; c < M; ++c) dot = fmaf(Ar[c], P2[i][c], dot);
+                float sl = 0.f;
+                fl += phi_one<GRAD>(B, br - dot, sl);
+                if (GRAD) {
+#pragma unroll
+                    for (int c = 0; c < M; ++c) df[i][c] = fmaf(-sl, Ar[c], df[i][c]);
+                }
+            }
+        }
+    }
+    s_red[0][tid] = fmaf(mu, fl, loss);
+    s_red[1][tid] = dT;
+    __syncthreads();
+    if (act) {
+        if (GRAD) {  // each interior point by one thread
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int c = 0; c < M; ++c) sG[q * PS + (2 * a + 1 + i) * M + c] += df[i][c] * (mu * up);
+        }
+        if (a == 0) {
+            float v = 0.f, w = 0.f;
+#pragma unroll
+            for (int c = 0; c < M; ++c) {
+                v += s_red[0][tid + c];
+                w += s_red[1][tid + c];
+            }
+            if (R.loss) R.loss[s0 + q] = v;
+            if (GRAD) R.dT[s0 + q] = w * up;
+        }
+    }
     if (GRAD) {
-#pragma unroll
-        for (int l = 1; l < PD; ++l)
-#pragma unroll
-            for (int a = 0; a < M; ++a) dPs[l * M + a] += df[l][a];
-        R.dT[s] = dT;
+        __syncthreads();
+        for (int u = tid; u < ns * L * M; u += NT) R.dP[s0 * L * M + u] = sG[u / (L * M) * PS + u % (L * M)];
     }
 }
 
@@ -211,15 +298,15 @@ bool refine_supported(int m, int g, int p) { return (m == 3 && g == 3 && p == 7)
 
 int launch_refine(const RefineParams& R, void* stream, int* launches) {
     cudaStream_t st = (cudaStream_t)stream;
-    const unsigned nb = (unsigned)((R.S + 127) / 128);
+    const unsigned nb = (unsigned)((R.S + RF_SEGS - 1) / RF_SEGS);
     if (R.S == 0) return 0;
     const bool grad = R.grad_loss != nullptr;
     if (R.m == 3 && R.g == 3 && R.p == 7) {
-        if (grad) k_refine<3, 3, 7, true><<<nb, 128, 0, st>>>(R);
-        else k_refine<3, 3, 7, false><<<nb, 128, 0, st>>>(R);
+        if (grad) k_refine<3, 3, 7, true><<<nb, RF_SEGS * 3, 0, st>>>(R);
+        else k_refine<3, 3, 7, false><<<nb, RF_SEGS * 3, 0, st>>>(R);
     } else if (R.m == 2 && R.g == 2 && R.p == 5) {
-        if (grad) k_refine<2, 2, 5, true><<<nb, 128, 0, st>>>(R);
-        else k_refine<2, 2, 5, false><<<nb, 128, 0, st>>>(R);
+        if (grad) k_refine<2, 2, 5, true><<<nb, RF_SEGS * 2, 0, st>>>(R);
+        else k_refine<2, 2, 5, false><<<nb, RF_SEGS * 2, 0, st>>>(R);
     } else {
         return (int)cudaErrorInvalidValue;
     }
