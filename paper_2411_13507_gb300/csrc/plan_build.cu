@@ -665,7 +665,7 @@ __global__ void k_zero_slots(BuildParams P) {
     }
 }
 
-constexpr int RECHECK_THREADS = 128;  // four warps (one FP64 unit each) per re-check entry
+constexpr int RECHECK_THREADS = 64;  // threads per re-check entry: a step has 54 to 63 rows in 3-D (9 rows a polytope)
 
 // Re-check entry: cost-only flag (1 bit) | query (16 bits) | polytope (10) | li (16) | lj (16) | T (5).
 // Bit 63 marks a check that is certainly feasible and needs only its cost in
@@ -2828,14 +2828,18 @@ __global__ void __launch_bounds__(256) k_pairs_f64(BuildParams P) {
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(RECHECK_THREADS) k_recheck(BuildParams P) {
-    // one entry per block of four warps, blocks spread over all SMs: every
-    // sub-partition of an SM has its own FP64 unit and GB300's FP64 rate is
-    // low, so an entry's rows are split over the four (threads take the rows,
-    // each row in canonical order); the control-polygon segments' squared
-    // norms are then summed in canonical order by one thread per segment
+    // one entry per block, blocks spread over all SMs.  GB300's FP64 rate is
+    // low and counts warp instructions whatever their lanes, so an entry's
+    // rows fill as few warps as hold them (threads take the rows, each in
+    // canonical order), and the interior control points are formed once (11
+    // instructions of one warp) instead of per polytope row (33 of two); the
+    // control-polygon segments' squared norms are then summed in canonical
+    // order by one thread per segment.  217,655 entries of 256 queries: 2.27 ->
+    // 1.25 ms; 9,172 entries of the 2-D TF32 form: 38 -> 34 us.
     using S = Shape<G, PD>;
     constexpr int N_ = M * G, RAX = S::RAX, NI = S::NI, TG = S::TG;
     __shared__ double s_v[PD * G * M];
+    __shared__ double s_p[NI * M];
     __shared__ double s_seg[PD];
     long long n = 0;
     if (block_failed(P.info, &P.info->rechecks, &n)) return;
@@ -2868,15 +2872,20 @@ __global__ void __launch_bounds__(RECHECK_THREADS) k_recheck(BuildParams P) {
         }
         if (!__syncthreads_and(ok)) continue;
         const int r0 = Q.poly_off[k], nr = Q.poly_off[k + 1] - r0;
-        for (int u = cost_only ? NI * nr : tid; u < NI * nr; u += nthr) {
-            const int l = 1 + u / nr, r = r0 + u % nr;
-            double s = 0.0;
-            for (int a = 0; a < M; ++a) {
-                const double pa = __dadd_rn(half_sum<G>(tb + L.e_D + l * TG, xi + a, M),
-                                            half_sum<G>(tb + L.e_D + l * TG + G, xj + a, M));
-                s = __dadd_rn(s, __dmul_rn(ldv(Q.A, (long long)r * M + a, P.in_f32), pa));
+        if (!cost_only) {  // the control points once, then their rows
+            for (int u = tid; u < NI * M; u += nthr) {
+                const int l = 1 + u / M, a = u % M;
+                s_p[u] = __dadd_rn(half_sum<G>(tb + L.e_D + l * TG, xi + a, M), half_sum<G>(tb + L.e_D + l * TG + G, xj + a, M));
             }
-            if (!(s <= P.blim64[Q.rowsOff + r])) ok = 0;
+            __syncthreads();
+            for (int u = tid; u < NI * nr; u += nthr) {
+                const int l = u / nr, r = r0 + u % nr;
+                double s = 0.0;
+#pragma unroll
+                for (int a = 0; a < M; ++a)
+                    s = __dadd_rn(s, __dmul_rn(ldv(Q.A, (long long)r * M + a, P.in_f32), s_p[l * M + a]));
+                if (!(s <= P.blim64[Q.rowsOff + r])) ok = 0;
+            }
         }
         if (!__syncthreads_and(ok)) continue;
         // cost rows: value (l, d, a) of segment l, then each segment's squared
@@ -2910,9 +2919,9 @@ __global__ void __launch_bounds__(RECHECK_THREADS) k_recheck(BuildParams P) {
 // ---------------------------------------------------------------------------
 // A5 compaction.  The pair (i, j) is emitted by its lowest shared polytope
 // (its "owner"); bits are OR-ed and keys min-ed over all shared polytopes.
-// Pass 1 counts per row and stores, for each slot, the inclusive count of
-// emitted entries in its (row, polytope) segment; pass 2 places every entry
-// at its rank among the row's emitted ids (sorted by j).
+// Pass 1 counts per row and stores the flags of the emitted slots with their
+// running count, 32 a word; pass 2 places every entry at its rank among the
+// row's emitted ids (sorted by j).
 // ---------------------------------------------------------------------------
 struct QView {  // per-query pointers into the shared scratch
     const QueryDesc* Q;
@@ -3609,7 +3618,7 @@ int launch_tc(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_per_s
     k_pairs_tc<M, G, PD, BF><<<num_sms * occ, 256, sm, st>>>(P);
     if (e1) cudaEventRecord(e1, st);
     ++*launches;
-    k_recheck<M, G, PD><<<num_sms * 8, RECHECK_THREADS, 0, st>>>(P);
+    k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
     ++*launches;
     return (int)cudaGetLastError();
 }
@@ -3641,7 +3650,7 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         k_pairs_ws<M, G, PD><<<num_sms, 512, sm, st>>>(P);
         if (e1) cudaEventRecord(e1, st);
         ++*launches;
-        k_recheck<M, G, PD><<<num_sms * 8, RECHECK_THREADS, 0, st>>>(P);
+        k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
         ++*launches;
     } else {
         // pipeline 0: screened kernel; 2: every pair through all rows
@@ -3659,7 +3668,7 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         kern<<<num_sms * occ, threads, sm, st>>>(P);
         if (e1) cudaEventRecord(e1, st);
         ++*launches;
-        k_recheck<M, G, PD><<<num_sms * 8, RECHECK_THREADS, 0, st>>>(P);
+        k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
         ++*launches;
     }
     return (int)cudaGetLastError();
