@@ -95,7 +95,8 @@ struct plan_ctx {
     long long want_slots = 0, want_rechecks = 0;
     uint32_t* resBits = nullptr;
     unsigned long long* resKey = nullptr;
-    int* emitPre = nullptr;
+    uint2* emit = nullptr;            // emitted flags (k_emit)
+    long long emitCap = 0;
     unsigned long long* recheck = nullptr;
     double* half64 = nullptr;         // FP64 cost halves of every state, duration and side (FP64 cost pass)
     float* half32 = nullptr;          // FP32 copy behind it (nullptr: no room)
@@ -323,7 +324,7 @@ int ensure_host_sized(plan_ctx* c, long long mask, long long list, long long k1,
 
 int ensure_device_sized(plan_ctx* c, long long slots, long long rechecks) {
     if (slots > c->slotCap) {
-        if (!dalloc(c, &c->resBits, slots) || !dalloc(c, &c->resKey, slots) || !dalloc(c, &c->emitPre, slots)) {
+        if (!dalloc(c, &c->resBits, slots) || !dalloc(c, &c->resKey, slots)) {
             c->slotCap = 0;
             return PLAN_ERR_NO_MEMORY;
         }
@@ -335,6 +336,18 @@ int ensure_device_sized(plan_ctx* c, long long slots, long long rechecks) {
             return PLAN_ERR_NO_MEMORY;
         }
         c->recheckCap = rechecks;
+    }
+    return PLAN_OK;
+}
+
+// Flags of the emitted slots: at most one entry per 32 slots and one per
+// membership, of which there are at most `list` and no more than slots.
+int ensure_emit(plan_ctx* c, long long list) {
+    const long long need = c->slotCap / 32 + (list < c->slotCap ? list : c->slotCap) + 2;
+    if (need > c->emitCap) {
+        c->emitCap = 0;
+        if (!dalloc(c, &c->emit, need)) return PLAN_ERR_NO_MEMORY;
+        c->emitCap = need;
     }
     return PLAN_OK;
 }
@@ -426,7 +439,7 @@ void plan_destroy(plan_ctx* c) {
     if (c->stream || c->d_info) cudaStreamSynchronize(c->stream);
     void* dev[] = {c->d_tab64, c->d_tab32, c->d_info, c->memMask, c->counts, c->members, c->localIdx, c->segKL, c->centers,
                    c->blim64, c->A32, c->blim32, c->bc32, c->resOff, c->itemOff, c->kPerm, c->ntile, c->tsize, c->iRange, c->rowCount,
-                   c->resBits, c->resKey, c->emitPre, c->recheck, c->half64, c->sdist, c->sbest, c->sbest16, c->spred, c->sfront, c->slast, c->snear,
+                   c->resBits, c->resKey, c->emit, c->recheck, c->half64, c->sdist, c->sbest, c->sbest16, c->spred, c->sfront, c->slast, c->snear,
                    c->d_qd, c->d_pfx, c->d_qSlot, c->d_qItem, c->d_qMem, c->d_rowRange, c->d_sqd, c->memOff,
                    c->d_cut64, c->d_cut32, c->cut_src, c->cut_hit, c->cut_pos, c->cut_chunk, c->cut_orow,
                    c->cut_ocount, c->cut_list32, c->cut_okb, c->cut_obox, c->pl_orow, c->pl_face, c->pl_edge, c->pl_nedge, c->pl_ocount, c->pl_keys, c->pl_near, c->pl_ub, c->d_mpc, c->d_mpcJ, c->g_d, c->g_succ, c->g_wsucc, c->g_anc, c->g_prev};
@@ -566,6 +579,8 @@ int prepare(plan_ctx* c, int Q, const plan_query* qs, int max_rows, int shard = 
     if (want_r == 0) want_r = 1 << 16;
     rc = ensure_device_sized(c, want_s, want_r);
     if (rc != PLAN_OK) return rc;
+    rc = ensure_emit(c, list);
+    if (rc != PLAN_OK) return rc;
     if (c->model.arith == PLAN_F64) {
         // the FP64 cost pass: both cost halves of every state and duration
         const int DR = c->model.cost_mode == PLAN_COST_POS ? 1 : c->model.gamma;
@@ -699,7 +714,7 @@ int issue(plan_ctx* c) {
     P.memOff = c->memOff;
     P.resBits = c->resBits;
     P.resKey = c->resKey;
-    P.emitPre = c->emitPre;
+    P.emit = c->emit;
     P.recheck = c->recheck;
     P.rowCount = c->rowCount;
     P.slotCap = c->slotCap;

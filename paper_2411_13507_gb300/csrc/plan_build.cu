@@ -210,6 +210,8 @@ __global__ void k_prep(BuildParams P) {
 // A1 membership: bit k of state i set iff A_k x_i^(0) <= b_k - eps on every
 // row (canonical FP64 decision; FP32 first, FP64 only inside the band).
 // ---------------------------------------------------------------------------
+// Few states: one warp per (state, word), a lane per polytope -- every lane's
+// rows are other lines, but no warp waits for more than one polytope's rows.
 DEVI void member_word(const BuildParams& P, long long t, int lane) {
     const int q = find_q(P.pfxMask, P.Q, t);
     const QueryDesc& Q = P.qd[q];
@@ -279,6 +281,102 @@ __global__ void __launch_bounds__(256, 4) k_member(BuildParams P) {
     for (long long t = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; t < P.totMask;
          t += ((long long)gridDim.x * blockDim.x) >> 5)
         member_word(P, t, lane);
+}
+
+// Many states: a CTA takes 256 consecutive states of a query (a thread each)
+// and the up to 32 polytopes of one mask word, whose rows it stages in shared
+// memory: a row is one broadcast load for a warp, and a warp leaves a polytope
+// once none of its states can be inside.  256 queries (1.2 M states, 8 to 128
+// polytopes): 2.33 -> 0.87 ms.  A warp's 32 polytopes follow one another, which
+// takes 16 to 34 us whatever the size, so a single query (5 us in 2-D, 16 us in
+// 3-D with a lane per polytope) keeps the form above: the many-states form
+// needs four CTAs an SM.
+constexpr int MEM_STATES = 256;
+
+// Items (MEM_STATES states, one word) of query q start at member_first(q): its
+// mask words so far over MEM_STATES, and room for each query's short last group
+// (N W / 256 + W items at most, W the widest query's).
+__host__ __device__ inline long long member_first(const BuildParams& P, long long mask, int q) {
+    return mask / MEM_STATES + (long long)q * (((P.maxK + 31) >> 5) + 2);
+}
+__host__ __device__ inline long long member_items(const BuildParams& P) { return member_first(P, P.totMask, P.Q); }
+
+__global__ void __launch_bounds__(MEM_STATES) k_member_many(BuildParams P) {
+    __shared__ float4 s_row[32 * RMAX];  // row r of polytope k at k * RMAX + r: A_r, and b_r in s_lim
+    __shared__ float s_lim[32 * RMAX];
+    __shared__ int s_n[32];              // rows of the polytope, -1: not a valid one
+    const int tid = threadIdx.x;
+    if (block_failed(P.info, nullptr, nullptr)) return;
+    const int m = P.m, n = P.m * P.g;
+    for (long long t = blockIdx.x; t < member_items(P); t += gridDim.x) {
+        int lo = 0, hi = P.Q;  // the query whose items t falls among
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (member_first(P, P.pfxMask[mid], mid) <= t) lo = mid;
+            else hi = mid;
+        }
+        const QueryDesc& Q = P.qd[lo];
+        const long long loc = t - member_first(P, P.pfxMask[lo], lo);
+        if (loc >= (long long)((Q.N + MEM_STATES - 1) / MEM_STATES) * Q.W) continue;
+        const int w = (int)(loc % Q.W), i = (int)(loc / Q.W) * MEM_STATES + tid;
+        const int k0 = w * 32, nk = min(32, Q.K - k0);
+        const int* poff = Q.poly_off;
+        __syncthreads();  // the previous item's rows are done with
+        for (int u = tid; u < nk * RMAX; u += MEM_STATES) {
+            const int k = u / RMAX, rr = u % RMAX, r0 = poff[k0 + k], nr = poff[k0 + k + 1] - r0;
+            const bool ok = nr >= 0 && nr <= P.max_rows && r0 >= 0 && r0 + nr <= Q.K * P.max_rows;
+            if (rr == 0) s_n[k] = ok ? nr : -1;
+            if (ok && rr < nr) {
+                const long long rg = Q.rowsOff + r0 + rr;
+                s_row[u] = make_float4(P.A32[rg * m], m > 1 ? P.A32[rg * m + 1] : 0.f, m > 2 ? P.A32[rg * m + 2] : 0.f,
+                                       m > 3 ? P.A32[rg * m + 3] : 0.f);
+                s_lim[u] = P.blim32[rg];
+            }
+        }
+        const bool valid = i < Q.N;
+        double x64[4];
+        float x32[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            x64[a] = a < m && valid ? ldv(Q.states, (long long)i * n + a, P.in_f32) : 0.0;
+            x32[a] = (float)x64[a];
+        }
+        __syncthreads();
+        uint32_t word = 0;
+        for (int k = 0; k < nk; ++k) {
+            const int nr = s_n[k];
+            bool in = valid && nr >= 0;
+            for (int r = 0; r < nr; ++r) {
+                const float4 A = s_row[k * RMAX + r];
+                const float lim = s_lim[k * RMAX + r];
+                const float av[4] = {A.x, A.y, A.z, A.w};
+                float s = 0.f, mag = 0.f;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    if (a < m) {
+                        s = fmaf(av[a], x32[a], s);
+                        mag = fmaf(fabsf(av[a]), fabsf(x32[a]), mag);
+                    }
+                }
+                const float d = s - lim;
+                const float band = KMEM * (mag + fabsf(lim));
+                if (in && !(d < -band)) {
+                    if (d > band) {
+                        in = false;
+                    } else {  // within the band (or NaN): canonical FP64 row
+                        const long long r0 = poff[k0 + k];
+                        double sd = 0.0;
+                        for (int a = 0; a < m; ++a)
+                            sd = __dadd_rn(sd, __dmul_rn(ldv(Q.A, (r0 + r) * m + a, P.in_f32), x64[a]));
+                        if (!(sd <= P.blim64[Q.rowsOff + r0 + r])) in = false;
+                    }
+                }
+                if ((r & 1) && !__any_sync(0xffffffffu, in)) break;
+            }
+            word |= in ? 1u << k : 0u;
+        }
+        if (valid) P.memMask[Q.maskOff + (long long)i * Q.W + w] = word;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2957,22 +3055,6 @@ DEVI int owner_of(const QView& V, int i, int j, int& nshared) {
     return owner;
 }
 
-DEVI void combine(const BuildParams& P, const QView& V, int i, int j, int k, uint32_t& bits, unsigned long long& key) {
-    const int W = V.Q->W;
-    for (int w = k >> 5; w < W; ++w) {
-        uint32_t x = V.mask[(long long)i * W + w] & V.mask[(long long)j * W + w];
-        if (w == (k >> 5)) x &= ~((2u << (k & 31)) - 1u);  // polytopes above k
-        while (x) {
-            const int k2 = w * 32 + __ffs(x) - 1;
-            x &= x - 1u;
-            const long long s2 = V.seg(k2, i) + V.localIdx[(long long)k2 * V.Q->N + j];
-            bits |= P.resBits[s2];
-            const unsigned long long k2v = P.resKey[s2];
-            if (k2v < key) key = k2v;
-        }
-    }
-}
-
 // Segment of the flat membership index g: query, polytope k and the state's
 // local index li in it.
 struct SegRef {
@@ -2987,72 +3069,189 @@ DEVI SegRef seg_of(const BuildParams& P, long long g) {
     return r;
 }
 
+// Emitted flags of a row segment g (slots base .. base + nk of polytope k):
+// per 32 slots a word of flags and the segment's count before it, in entries
+// base / 32 + g onwards (segments follow one another in slots and in g, so
+// they do not overlap: floor((base + nk) / 32) + 1 - floor(base / 32) >=
+// ceil(nk / 32)).
+DEVI long long emit_at(long long base, long long g) { return (base >> 5) + g; }
+
+// Emitted entries of a segment before its slot lj.
+DEVI int emit_rank(const uint2* em, int lj) {
+    const uint2 w = em[lj >> 5];
+    return (int)w.y + __popc(w.x & ((1u << (lj & 31)) - 1u));
+}
+
 // Pass 1, one warp per row segment (state i in polytope k, its slots (i, j)
 // for the polytope's members j): is each slot the pair's owner (the lowest
 // polytope both states contain -- only pairs of states that both lie in
 // several polytopes can be shared), and is the pair feasible for some
 // duration?  The owner slot receives the pair's result combined over all
-// shared polytopes; emitPre gets the inclusive prefix of the emitted flags
-// within the segment, and the segment total adds to row i's count.
+// shared polytopes; the segment's flags go to emit, its total to row i's
+// count.
+//
+// Bound by its instructions at a low issue rate (chains of dependent loads),
+// not by the 4 bytes of bits a slot needs.  A row of a state in one polytope
+// needs no ids at all; in the others the loads of four chunks of 32 slots and
+// of their membership words are issued together, and the pairs that combine
+// are gathered so that the lanes follow their chains of loads at the same time.
+// The flags are one bit a slot instead of a prefix of 4 bytes, and keys are
+// read only where results combine (256 queries, 451 M slots: 4.05 -> 2.84 ms).
 __global__ void __launch_bounds__(256, 4) k_emit(BuildParams P) {
+    __shared__ long long s_seg[8][32];  // slot of (i, member 0) in the row's t-th polytope
+    __shared__ uint32_t s_comb[8][128]; // combined bits of a group's slots
+    __shared__ uint8_t s_list[8][128];  // slots of a group whose results combine
     long long nseg = 0;
     if (block_failed(P.info, &P.info->memberships, &nseg)) return;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     unsigned long long cand = 0, chk = 0, feas = 0;
     for (long long g = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; g < nseg;
          g += ((long long)gridDim.x * blockDim.x) >> 5) {
         const SegRef sr = seg_of(P, g);
         const QView V(P, sr.q);
         const QueryDesc& Q = *V.Q;
-        const int k = sr.k, nk = V.counts[k];
+        const int k = sr.k, nk = V.counts[k], W = Q.W;
         const int* mem = V.members + (long long)k * Q.N;
         const int im = mem[sr.li];
         const int i = mem_id(im);
         if (i < P.rowRange[2 * sr.q] || i >= P.rowRange[2 * sr.q + 1]) continue;  // another shard's row
+        const bool multi = mem_multi(im);
         const long long base = V.slot0 + V.resOff[k] + (long long)sr.li * nk;
-        int running = 0;
+        const uint32_t mi = multi && lane < W ? V.mask[(long long)i * W + lane] : 0u;  // lane w: word w of row i (W <= 32)
+        uint2* em = P.emit + emit_at(base, g);
+        int running = 0, nfeas = 0;
+        if (!multi) {  // the owner of all its pairs; the pair (i, i) has no bits
+            for (int lg = 0; lg < nk; lg += 128) {
+                uint32_t bv[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int lj = lg + 32 * c + lane;
+                    bv[c] = lj < nk ? P.resBits[base + lj] : 0u;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (lg + 32 * c >= nk) break;  // warp-uniform
+                    const unsigned bal = __ballot_sync(0xffffffffu, bv[c] != 0);
+                    nfeas += __popc(bv[c]);
+                    if (lane == 0) em[(lg >> 5) + c] = make_uint2(bal, (unsigned)running);
+                    running += __popc(bal);
+                }
+            }
+            feas += nfeas;
+            if (lane == 0) {
+                cand += nk - 1;
+                chk += (unsigned long long)(nk - 1) * Q.nT;
+                if (running) atomicAdd(&P.rowCount[Q.rowOff + i], running);
+            }
+            continue;
+        }
+        bool looked_up = false;
+        int ncand = 0;
         for (int lg = 0; lg < nk; lg += 128) {
-            // four chunks of 32 slots: every load of the group is issued first
             int jv[4];
             uint32_t bv[4];
-            unsigned long long kv[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int lj = lg + 32 * c + lane;
                 const bool in = lj < nk;
-                jv[c] = in ? mem[lj] : 0;
+                jv[c] = in ? mem[lj] : i;  // no pair with itself (and without the flag of several polytopes)
                 bv[c] = in ? P.resBits[base + lj] : 0u;
-                kv[c] = in ? P.resKey[base + lj] : 0ull;
+            }
+            int owner[4], ns[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                owner[c] = k;
+                ns[c] = 1;
+            }
+            if (__any_sync(0xffffffffu, mem_multi(jv[0]) || mem_multi(jv[1]) || mem_multi(jv[2]) || mem_multi(jv[3]))) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (mem_multi(jv[c])) {
+                        owner[c] = -1;
+                        ns[c] = 0;
+                    }
+                for (int w = 0; w < W; ++w) {
+                    const uint32_t miw = __shfl_sync(0xffffffffu, mi, w);
+                    if (!miw) continue;
+                    uint32_t x[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) x[c] = mem_multi(jv[c]) ? V.mask[(long long)mem_id(jv[c]) * W + w] & miw : 0u;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        if (x[c] && owner[c] < 0) owner[c] = w * 32 + __ffs(x[c]) - 1;
+                        ns[c] += __popc(x[c]);
+                    }
+                }
+            }
+            // the pairs whose results combine, gathered so that lanes take them together
+            int ncomb = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const bool comb = mem_id(jv[c]) != i && owner[c] == k && ns[c] > 1;
+                const unsigned cb = __ballot_sync(0xffffffffu, comb);
+                if (comb) s_list[wib][ncomb + __popc(cb & ((1u << lane) - 1u))] = (uint8_t)(32 * c + lane);
+                ncomb += __popc(cb);
+            }
+            if (ncomb > 0) {
+                if (!looked_up) {  // slot of (i, member 0) in the row's t-th polytope, t < 32
+                    looked_up = true;
+                    int before = 0;
+                    for (int w = 0; w < W; ++w) {
+                        const uint32_t miw = __shfl_sync(0xffffffffu, mi, w);
+                        if ((miw >> lane) & 1u) {
+                            const int t = before + __popc(miw & ((1u << lane) - 1u));
+                            if (t < 32) s_seg[wib][t] = V.seg(w * 32 + lane, i);
+                        }
+                        before += __popc(miw);
+                    }
+                }
+                __syncwarp();
+                for (int e = lane; e < ncomb; e += 32) {
+                    const int u = s_list[wib][e], j = mem_id(mem[lg + u]);
+                    const long long slot = base + lg + u;
+                    uint32_t bits = P.resBits[slot];
+                    unsigned long long key = P.resKey[slot];
+                    int before = 0;
+                    for (int w = 0; w < W; ++w) {
+                        const uint32_t miw = V.mask[(long long)i * W + w];
+                        uint32_t x = miw & V.mask[(long long)j * W + w];
+                        if (w == (k >> 5)) x &= ~((2u << (k & 31)) - 1u);  // polytopes above k
+                        else if (w < (k >> 5)) x = 0u;
+                        while (x) {
+                            const int bit = __ffs(x) - 1, k2 = w * 32 + bit;
+                            x &= x - 1u;
+                            const int t = before + __popc(miw & ((1u << bit) - 1u));
+                            const long long s2 = (t < 32 ? s_seg[wib][t] : V.seg(k2, i)) + V.localIdx[(long long)k2 * Q.N + j];
+                            bits |= P.resBits[s2];
+                            const unsigned long long k2v = P.resKey[s2];
+                            if (k2v < key) key = k2v;
+                        }
+                        before += __popc(miw);
+                    }
+                    P.resBits[slot] = bits;
+                    P.resKey[slot] = key;
+                    s_comb[wib][u] = bits;
+                }
+                __syncwarp();
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const int lj = lg + 32 * c + lane;
                 if (lg + 32 * c >= nk) break;  // warp-uniform
-                int flag = 0;
-                if (lj < nk) {
-                    const int jm = jv[c], j = mem_id(jm);
-                    if (i != j) {
-                        int ns = 1;
-                        if (!(mem_multi(im) && mem_multi(jm)) || owner_of(V, i, j, ns) == k) {
-                            ++cand;
-                            chk += Q.nT;
-                            uint32_t bits = bv[c];
-                            if (ns > 1) {
-                                unsigned long long key = kv[c];
-                                combine(P, V, i, j, k, bits, key);
-                                P.resBits[base + lj] = bits;
-                                P.resKey[base + lj] = key;
-                            }
-                            flag = bits != 0;
-                            feas += __popc(bits);
-                        }
-                    }
+                const bool own = mem_id(jv[c]) != i && owner[c] == k;
+                const uint32_t bits = own && ns[c] > 1 ? s_comb[wib][32 * c + lane] : bv[c];
+                if (own) {
+                    ++ncand;
+                    nfeas += __popc(bits);
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, flag != 0);
-                if (lj < nk) P.emitPre[base + lj] = running + __popc(bal & ((2u << lane) - 1u));
+                const unsigned bal = __ballot_sync(0xffffffffu, own && bits != 0);
+                if (lane == 0) em[(lg >> 5) + c] = make_uint2(bal, (unsigned)running);
                 running += __popc(bal);
             }
+            __syncwarp();  // the list and the bits are rewritten by the next group
         }
+        cand += ncand;
+        chk += (unsigned long long)ncand * Q.nT;
+        feas += nfeas;
         if (lane == 0 && running) atomicAdd(&P.rowCount[Q.rowOff + i], running);
     }
     block_add(&P.info->candidates, cand);
@@ -3096,69 +3295,66 @@ DEVI void write_edge(const BuildParams& P, const QueryDesc& Q, long long o, int 
     else ((float*)Q.w)[o] = __uint_as_float((unsigned)(key >> 32));
 }
 
-// Output pass.  Work items [0, memberships) are row segments: a state that
-// lies in one polytope only has its whole row there, so an emitted entry's
-// rank in the row is the segment prefix -- one warp per segment.  Items
-// [memberships, memberships + rows) are rows of states in several polytopes:
-// one warp per row merges its segments' emitted ids (each segment already in
-// ascending order) by rank, with the segments' ids staged in shared memory,
-// or, when they do not fit, by binary searches in the other segments' member
-// lists.
+// Output pass, one warp per row segment: a state that lies in one polytope
+// only has its whole row there, so an emitted entry's rank in the row is the
+// segment's running count.  A row of a state in several polytopes goes with its
+// segment of the lowest one, whose warp merges the row's segments' emitted ids
+// (each already in ascending order) by rank, with the ids staged in shared
+// memory, or, when they do not fit, by binary searches in the other segments'
+// member lists.
 __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_cap) {
     extern __shared__ uint32_t bmem[];
     __shared__ int s_meta[8][32 * 4 + 1];
-    __shared__ long long s_metab[8][32];
+    __shared__ long long s_metab[8][2 * 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     long long nseg = 0;
     if (block_failed(P.info, &P.info->memberships, &nseg)) return;
-    const long long nitem = nseg + P.totN;
     int* runs = reinterpret_cast<int*>(bmem) + (size_t)wib * run_cap;  // this warp's staged ids
-    for (long long it0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; it0 < nitem;
-         it0 += ((long long)gridDim.x * blockDim.x) >> 5) {
-        // rows first: the long multi-polytope rows start early instead of
-        // forming the tail
-        const long long it = it0 < P.totN ? nseg + it0 : it0 - P.totN;
-        if (it < nseg) {
-            const SegRef sr = seg_of(P, it);
-            const QView V(P, sr.q);
-            const QueryDesc& Q = *V.Q;
+    for (long long it = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; it < nseg;
+         it += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const SegRef sr = seg_of(P, it);
+        const int q = sr.q;
+        const QView V(P, q);
+        const QueryDesc& Q = *V.Q;
+        const int im = (V.members + (long long)sr.k * Q.N)[sr.li], i = mem_id(im);
+        if (i < P.rowRange[2 * q] || i >= P.rowRange[2 * q + 1]) continue;  // another shard's row
+        if (!mem_multi(im)) {
             const int* mem = V.members + (long long)sr.k * Q.N;
-            const int im = mem[sr.li];
-            if (mem_multi(im)) continue;  // the row item handles it
-            if (mem_id(im) < P.rowRange[2 * sr.q] || mem_id(im) >= P.rowRange[2 * sr.q + 1]) continue;
             const int nk = V.counts[sr.k];
             const long long base = V.slot0 + V.resOff[sr.k] + (long long)sr.li * nk;
-            const long long rbase = Q.row_off[mem_id(im)];
+            const long long rbase = Q.row_off[i];
+            const uint2* em = P.emit + emit_at(base, it);
             for (int lg = 0; lg < nk; lg += 128) {
-                int pv[4], pp[4], jv[4];
+                uint2 ew[4];
+                int jv[4];
                 uint32_t bv[4];
                 unsigned long long kv[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {  // every load of the group first
+                for (int c = 0; c < 4; ++c) ew[c] = lg + 32 * c < nk ? em[(lg >> 5) + c] : make_uint2(0u, 0u);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {  // every load of the group first, of emitted slots only
                     const int lj = lg + 32 * c + lane;
-                    const bool in = lj < nk;
-                    pv[c] = in ? P.emitPre[base + lj] : 0;
-                    pp[c] = in && lj > 0 ? P.emitPre[base + lj - 1] : 0;
+                    const bool in = (ew[c].x >> lane) & 1u;
                     jv[c] = in ? mem[lj] : 0;
                     bv[c] = in ? P.resBits[base + lj] : 0u;
                     kv[c] = in ? P.resKey[base + lj] : 0ull;
                 }
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (pv[c] != pp[c]) write_edge(P, Q, rbase + pp[c], mem_id(jv[c]), bv[c], kv[c]);
+                    if ((ew[c].x >> lane) & 1u)
+                        write_edge(P, Q, rbase + (int)ew[c].y + __popc(ew[c].x & ((1u << lane) - 1u)), mem_id(jv[c]), bv[c], kv[c]);
             }
             continue;
         }
-        const long long row = it - nseg;
-        const int q = find_q(P.pfxN, P.Q, row);
-        const QView V(P, q);
-        const QueryDesc& Q = *V.Q;
-        const int i = (int)(row - P.pfxN[q]);
-        if (i < P.rowRange[2 * q] || i >= P.rowRange[2 * q + 1]) continue;  // another shard's row
+        // a row of several polytopes: with its segment of the lowest one
         const int W = Q.W;
-        int npoly = 0;
-        for (int w = 0; w < W; ++w) npoly += __popc(V.mask[(long long)i * W + w]);
-        if (npoly < 2) continue;  // a segment item handled it
+        int npoly = 0, first = -1;
+        for (int w = 0; w < W; ++w) {
+            const uint32_t mw = V.mask[(long long)i * W + w];
+            if (mw && first < 0) first = w * 32 + __ffs(mw) - 1;
+            npoly += __popc(mw);
+        }
+        if (first != sr.k) continue;
         const long long rbase = Q.row_off[i];
         // Segment metadata (lane t: the row's t-th polytope): base slot, size,
         // emitted count (the segment prefix at its last slot), run offset.
@@ -3167,6 +3363,7 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
         int* s_e = s_k + 64;
         int* s_off = s_k + 96;  // 33 entries
         long long* s_base = s_metab[wib];
+        long long* s_em = s_base + 32;  // entries of its flags
         int total = 0x7fffffff;
         if (npoly <= 32) {
             if (lane == 0) {
@@ -3181,11 +3378,13 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
             }
             __syncwarp();
             if (lane < npoly) {
-                const int k = s_k[lane], nk = V.counts[k];
-                const long long base = V.seg(k, i);
+                const int k = s_k[lane], nk = V.counts[k], li = V.localIdx[(long long)k * Q.N + i];
+                const long long base = V.slot0 + V.resOff[k] + (long long)li * nk;
+                const long long at = emit_at(base, P.qMem[q] + P.memOff[Q.kOff + k] + li);
                 s_nk[lane] = nk;
                 s_base[lane] = base;
-                s_e[lane] = nk > 0 ? P.emitPre[base + nk - 1] : 0;
+                s_em[lane] = at;
+                s_e[lane] = nk > 0 ? emit_rank(P.emit + at, nk - 1) + (int)((P.emit[at + ((nk - 1) >> 5)].x >> ((nk - 1) & 31)) & 1u) : 0;
             }
             __syncwarp();
             if (lane == 0) {
@@ -3207,24 +3406,24 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
             int* runj = runs + run_cap / 2;  // slot index (within its segment) of each staged id
             for (int t = 0; t < npoly; ++t) {
                 const int nk = s_nk[t];
-                const long long base = s_base[t];
                 const int* mem = V.members + (long long)s_k[t] * Q.N;
                 const int off = s_off[t];
+                const uint2* em = P.emit + s_em[t];
                 for (int lg = 0; lg < nk; lg += 128) {
-                    int pv[4], pp[4], jv[4];
+                    uint2 ew[4];
+                    int jv[4];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {  // every load of the group first
                         const int lj = lg + 32 * c + lane;
-                        const bool in = lj < nk;
-                        pv[c] = in ? P.emitPre[base + lj] : 0;
-                        pp[c] = in && lj > 0 ? P.emitPre[base + lj - 1] : 0;
-                        jv[c] = in ? mem[lj] : 0;
+                        ew[c] = lg + 32 * c < nk ? em[(lg >> 5) + c] : make_uint2(0u, 0u);
+                        jv[c] = lj < nk ? mem[lj] : 0;
                     }
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        if (pv[c] != pp[c]) {
-                            runs[off + pp[c]] = mem_id(jv[c]);
-                            runj[off + pp[c]] = lg + 32 * c + lane;
+                        if ((ew[c].x >> lane) & 1u) {
+                            const int r = off + (int)ew[c].y + __popc(ew[c].x & ((1u << lane) - 1u));
+                            runs[r] = mem_id(jv[c]);
+                            runj[r] = lg + 32 * c + lane;
                         }
                 }
             }
@@ -3279,24 +3478,25 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
                 while (mw) {
                     const int k = w * 32 + __ffs(mw) - 1;
                     mw &= mw - 1u;
-                    const int nk = V.counts[k];
-                    const long long base = V.seg(k, i);
+                    const int nk = V.counts[k], li = V.localIdx[(long long)k * Q.N + i];
+                    const long long base = V.slot0 + V.resOff[k] + (long long)li * nk;
+                    const uint2* em = P.emit + emit_at(base, P.qMem[q] + P.memOff[Q.kOff + k] + li);
                     const int* mem = V.members + (long long)k * Q.N;
                     for (int lj = lane; lj < nk; lj += 32) {
-                        const int pre = P.emitPre[base + lj];
-                        const int prev = lj > 0 ? P.emitPre[base + lj - 1] : 0;
-                        if (pre == prev) continue;  // not emitted here
+                        if (!((em[lj >> 5].x >> (lj & 31)) & 1u)) continue;  // not emitted here
                         const int j = mem_id(mem[lj]);
-                        long long rank = prev;
+                        long long rank = emit_rank(em, lj);
                         for (int w2 = 0; w2 < W; ++w2) {
                             uint32_t m2 = V.mask[(long long)i * W + w2];
                             while (m2) {
                                 const int k2 = w2 * 32 + __ffs(m2) - 1;
                                 m2 &= m2 - 1u;
                                 if (k2 == k) continue;
-                                const int n2 = V.counts[k2];
+                                const int n2 = V.counts[k2], l2 = V.localIdx[(long long)k2 * Q.N + i];
                                 const int pos = lower_bound_members(V.members + (long long)k2 * Q.N, n2, j);
-                                if (pos > 0) rank += P.emitPre[V.seg(k2, i) + pos - 1];
+                                const long long b2 = V.slot0 + V.resOff[k2] + (long long)l2 * n2;
+                                const uint2* e2 = P.emit + emit_at(b2, P.qMem[q] + P.memOff[Q.kOff + k2] + l2);
+                                if (pos > 0) rank += emit_rank(e2, pos - 1) + (int)((e2[(pos - 1) >> 5].x >> ((pos - 1) & 31)) & 1u);
                             }
                         }
                         write_edge(P, Q, rbase + rank, j, P.resBits[base + lj], P.resKey[base + lj]);
@@ -3705,8 +3905,11 @@ int launch_build(const BuildParams& P, void* stream, int num_sms, int ctas_per_s
         ++*launches;
     }
     if (P.totMask > 0) {  // also writes the (zero) masks of queries without polytopes
-        const long long need = (P.totMask * 32 + 255) / 256;
-        k_member<<<(unsigned)(need < num_sms * 4 ? need : num_sms * 4), 256, 0, st>>>(P);
+        const long long many = member_items(P), need = (P.totMask * 32 + 255) / 256;
+        if (many >= 4LL * num_sms)
+            k_member_many<<<(unsigned)(many < num_sms * 8 ? many : num_sms * 8), MEM_STATES, 0, st>>>(P);
+        else
+            k_member<<<(unsigned)(need < num_sms * 4 ? need : num_sms * 4), 256, 0, st>>>(P);
         ++*launches;
     }
     if (P.totPoly > 0) {

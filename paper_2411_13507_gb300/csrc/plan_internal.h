@@ -3,6 +3,8 @@
 
 #include <cstdint>
 
+#include <vector_types.h>
+
 #include "../../include/plan.h"
 
 namespace plan {
@@ -179,7 +181,7 @@ struct BuildParams {
     int* rowRange;             // [Q][2] row range [lo, hi) of each query's shard (written by k_setup)
     uint32_t* resBits;
     unsigned long long* resKey;
-    int* emitPre;
+    uint2* emit;               // emitted flags of 32 slots of a segment and the count before them (emit_at)
     unsigned long long* recheck;
     int* rowCount;
     long long slotCap, recheckCap;
