@@ -185,6 +185,7 @@ DEVI int find_q(const long long* pfx, int Q, long long x) {
 // Rows of every polytope: FP32 copies, b - eps, row-count checks.
 // ---------------------------------------------------------------------------
 __global__ void k_prep(BuildParams P) {
+    after_stream<true>();
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= P.totRows) return;
     const int q = find_q(P.pfxRows, P.Q, t);
@@ -274,6 +275,7 @@ DEVI void member_word(const BuildParams& P, long long t, int lane) {
 }
 
 __global__ void __launch_bounds__(256, 4) k_member(BuildParams P) {
+    after_stream<true>();
     const int lane = threadIdx.x & 31;
     if (block_failed(P.info, nullptr, nullptr)) return;
     // one warp per (state, word), persistent: a single wave of CTAs loops
@@ -302,6 +304,7 @@ __host__ __device__ inline long long member_first(const BuildParams& P, long lon
 __host__ __device__ inline long long member_items(const BuildParams& P) { return member_first(P, P.totMask, P.Q); }
 
 __global__ void __launch_bounds__(MEM_STATES) k_member_many(BuildParams P) {
+    after_stream<false>();
     __shared__ float4 s_row[32 * RMAX];  // row r of polytope k at k * RMAX + r: A_r, and b_r in s_lim
     __shared__ float s_lim[32 * RMAX];
     __shared__ int s_n[32];              // rows of the polytope, -1: not a valid one
@@ -384,6 +387,7 @@ __global__ void __launch_bounds__(MEM_STATES) k_member_many(BuildParams P) {
 // block centre (first member's position) and centred FP32 bounds.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_lists(BuildParams P) {
+    after_stream<true>();
     const int q = find_q(P.pfxPoly, P.Q, blockIdx.x);
     const QueryDesc& Q = P.qd[q];
     const int k = (int)(blockIdx.x - P.pfxPoly[q]);
@@ -546,6 +550,7 @@ DEVI void shard_rows(const BuildParams& P, const QueryDesc& Q, int* s_counts, lo
 // block; the i-tiles cover only the members whose ids lie in the row range
 // (a contiguous part of the ascending member list), the j-tiles all members.
 __global__ void __launch_bounds__(1024) k_setup(BuildParams P) {
+    after_stream<true>();
     __shared__ long long wb[32];
     __shared__ long long tot;
     __shared__ int s_counts[1024];
@@ -638,6 +643,7 @@ __global__ void __launch_bounds__(1024) k_setup(BuildParams P) {
 
 // Prefix sums of the per-query slot and tile totals; scratch capacity check.
 __global__ void __launch_bounds__(1024) k_batch(BuildParams P) {
+    after_stream<true>();
     __shared__ long long wb[32];
     __shared__ long long tot;
     long long cs = 0, ci = 0, cm = 0;
@@ -742,15 +748,18 @@ DEVI ItemT item_decode_chunk(const BuildParams& P, long long item) {
 
 // Slots start empty (no feasible duration, no key); the pair kernels merge
 // into them with atomics.
-// Clears the pair slots and writes the row-segment table (segment g -> its
+// Clears the pair slots and row counts and writes the row-segment table (segment g -> its
 // polytope and local index), one warp per polytope.
 __global__ void k_zero_slots(BuildParams P) {
+    after_stream<false>();
     long long n = 0;
     if (block_failed(P.info, &P.info->slots, &n)) return;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
         P.resBits[s] = 0u;
         P.resKey[s] = KEY_NONE;
     }
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P.totN; i += (long long)gridDim.x * blockDim.x)
+        P.rowCount[i] = 0;
     const int lane = threadIdx.x & 31;
     for (long long gp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; gp < P.totPoly;
          gp += ((long long)gridDim.x * blockDim.x) >> 5) {
@@ -1054,6 +1063,7 @@ DEVI void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory");
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256, 2) k_pairs_fast(BuildParams P) {
+    after_stream<false>();
     using S = Shape<G, PD>;
     using PT = PadTab<G, PD>;
     constexpr int N_ = M * G, RAX = S::RAX, RR = M * RAX, NI = S::NI;
@@ -1638,6 +1648,7 @@ constexpr int SC_STAGE = 160;
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
+    after_stream<false>();
     using S = Shape<G, PD>;
     using PT = PadTab<G, PD>;
     using SS = ScShape<M, G, PD>;
@@ -2085,6 +2096,7 @@ DEVI void bar_producers() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(512, 1) k_pairs_ws(BuildParams P) {
+    after_stream<false>();
     using S = Shape<G, PD>;
     constexpr int N_ = M * G, RAX = S::RAX, RR = M * RAX, NI = S::NI, TG = S::TG;
     constexpr int T = TILE;
@@ -2458,6 +2470,7 @@ DEVI uint32_t idesc(int Mdim, int Ndim, bool bf) {
 
 template <int M, int G, int PD, bool BF>
 __global__ void __launch_bounds__(256, 2) k_pairs_tc(BuildParams P) {
+    after_stream<false>();
     using S = Shape<G, PD>;
     constexpr int N_ = M * G, RAX = S::RAX, RR = M * RAX, NI = S::NI, TG = S::TG;
     constexpr int KFEAT = N_ + 1;
@@ -2776,6 +2789,7 @@ DEVI int reach_order(int r) {  // derivative order k of canonical reach row r (k
 // order, so no re-check is needed.
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256) k_pairs_f64(BuildParams P) {
+    after_stream<false>();
     using S = Shape<G, PD>;
     constexpr int N_ = M * G, RAX = S::RAX, RR = M * RAX, NI = S::NI, TG = S::TG;
     constexpr int T = TILE64;
@@ -2926,6 +2940,7 @@ __global__ void __launch_bounds__(256) k_pairs_f64(BuildParams P) {
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(RECHECK_THREADS) k_recheck(BuildParams P) {
+    after_stream<false>();
     // one entry per block, blocks spread over all SMs.  GB300's FP64 rate is
     // low and counts warp instructions whatever their lanes, so an entry's
     // rows fill as few warps as hold them (threads take the rows, each in
@@ -3098,6 +3113,7 @@ DEVI int emit_rank(const uint2* em, int lj) {
 // The flags are one bit a slot instead of a prefix of 4 bytes, and keys are
 // read only where results combine (256 queries, 451 M slots: 4.05 -> 2.84 ms).
 __global__ void __launch_bounds__(256, 4) k_emit(BuildParams P) {
+    after_stream<false>();
     __shared__ long long s_seg[8][32];  // slot of (i, member 0) in the row's t-th polytope
     __shared__ uint32_t s_comb[8][128]; // combined bits of a group's slots
     __shared__ uint8_t s_list[8][128];  // slots of a group whose results combine
@@ -3261,6 +3277,7 @@ __global__ void __launch_bounds__(256, 4) k_emit(BuildParams P) {
 
 // One CTA per query: exclusive scan of the row counts into row_off, E, capacity.
 __global__ void __launch_bounds__(1024) k_scan(BuildParams P) {
+    after_stream<true>();
     __shared__ long long wb[32];
     __shared__ long long tot;
     if (has_failed(P.info)) return;
@@ -3303,6 +3320,7 @@ DEVI void write_edge(const BuildParams& P, const QueryDesc& Q, long long o, int 
 // memory, or, when they do not fit, by binary searches in the other segments'
 // member lists.
 __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_cap) {
+    after_stream<false>();
     extern __shared__ uint32_t bmem[];
     __shared__ int s_meta[8][32 * 4 + 1];
     __shared__ long long s_metab[8][2 * 32];
@@ -3528,6 +3546,7 @@ __global__ void __launch_bounds__(256, 4) k_compact_fill(BuildParams P, int run_
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256) k_halves64(BuildParams P) {
+    after_stream<false>();
     constexpr int N_ = M * G, TG = 2 * G;
     if (block_failed(P.info, nullptr, nullptr)) return;
     const TabLayout L = P.L;
@@ -3595,6 +3614,7 @@ DEVI uint32_t cheapest_bits(uint32_t bits, const float* hl, const float* hr, int
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256) k_cost64(BuildParams P) {
+    after_stream<false>();
     if (block_failed(P.info, nullptr, nullptr)) return;
     const int DR = P.cost_mode == 1 ? 1 : G;
     const int E = PD * DR * M;
@@ -3815,10 +3835,10 @@ int launch_tc(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_per_s
     if (occ > 2) occ = 2;  // two 256-column tensor-memory allocations per SM
     if (ctas_per_sm > 0 && ctas_per_sm < occ) occ = ctas_per_sm;
     if (e0) cudaEventRecord(e0, st);
-    k_pairs_tc<M, G, PD, BF><<<num_sms * occ, 256, sm, st>>>(P);
+    launch_next(k_pairs_tc<M, G, PD, BF>, dim3(num_sms * occ), dim3(256), sm, st, P);
     if (e1) cudaEventRecord(e1, st);
     ++*launches;
-    k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
+    launch_next(k_recheck<M, G, PD>, dim3(num_sms * 16), dim3(RECHECK_THREADS), 0, st, P);
     ++*launches;
     return (int)cudaGetLastError();
 }
@@ -3840,17 +3860,17 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_f64<M, G, PD>, 256, sm);
         if (occ < 1) occ = 1;
         if (e0) cudaEventRecord(e0, st);
-        k_pairs_f64<M, G, PD><<<num_sms * occ, 256, sm, st>>>(P);
+        launch_next(k_pairs_f64<M, G, PD>, dim3(num_sms * occ), dim3(256), sm, st, P);
         if (e1) cudaEventRecord(e1, st);
         ++*launches;
     } else if (P.pipeline == 1 && P.tile == TILE && smem_ws<M, G, PD>(P) <= 227 * 1024) {
         const size_t sm = smem_ws<M, G, PD>(P);
         cudaFuncSetAttribute(k_pairs_ws<M, G, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e0) cudaEventRecord(e0, st);
-        k_pairs_ws<M, G, PD><<<num_sms, 512, sm, st>>>(P);
+        launch_next(k_pairs_ws<M, G, PD>, dim3(num_sms), dim3(512), sm, st, P);
         if (e1) cudaEventRecord(e1, st);
         ++*launches;
-        k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
+        launch_next(k_recheck<M, G, PD>, dim3(num_sms * 16), dim3(RECHECK_THREADS), 0, st, P);
         ++*launches;
     } else {
         // pipeline 0: screened kernel; 2: every pair through all rows
@@ -3865,10 +3885,10 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         if (occ < 1) occ = 1;
         if (ctas_per_sm > 0 && ctas_per_sm < occ) occ = ctas_per_sm;
         if (e0) cudaEventRecord(e0, st);
-        kern<<<num_sms * occ, threads, sm, st>>>(P);
+        launch_next(kern, dim3(num_sms * occ), dim3(threads), sm, st, P);
         if (e1) cudaEventRecord(e1, st);
         ++*launches;
-        k_recheck<M, G, PD><<<num_sms * 16, RECHECK_THREADS, 0, st>>>(P);
+        launch_next(k_recheck<M, G, PD>, dim3(num_sms * 16), dim3(RECHECK_THREADS), 0, st, P);
         ++*launches;
     }
     return (int)cudaGetLastError();
@@ -3887,12 +3907,12 @@ int launch_cost64(const BuildParams& P, cudaStream_t st, int num_sms) {
     const int DR = P.cost_mode == 1 ? 1 : G;
     const long long n = P.totN * (long long)P.maxT * 2 * PD * DR * M;
     const long long hb = (n + 255) / 256;
-    k_halves64<M, G, PD><<<(unsigned)(hb < (long long)num_sms * 8 ? (hb > 0 ? hb : 1) : (long long)num_sms * 8), 256, 0, st>>>(P);
+    launch_next(k_halves64<M, G, PD>, dim3((unsigned)(hb < (long long)num_sms * 8 ? (hb > 0 ? hb : 1) : (long long)num_sms * 8)), dim3(256), 0, st, P);
     // blocks per query: about eight two-warp CTAs per SM over the batch, at
     // least one; small CTAs spread a small graph's edges over every SM's
     // FP64 units (the CTAs past the edges exit at once)
     const int bx = (int)((long long)num_sms * 8 / P.Q > 0 ? (long long)num_sms * 8 / P.Q : 1);
-    k_cost64<M, G, PD><<<dim3((unsigned)bx, (unsigned)P.Q), 64, 0, st>>>(P);
+    launch_next(k_cost64<M, G, PD>, dim3((unsigned)bx, (unsigned)P.Q), dim3(64), 0, st, P);
     return (int)cudaGetLastError();
 }
 
@@ -3901,26 +3921,26 @@ int launch_build(const BuildParams& P, void* stream, int num_sms, int ctas_per_s
     cudaEvent_t e0 = (cudaEvent_t)ev0, e1 = (cudaEvent_t)ev1;
     if (P.Q <= 0) return 0;
     if (P.totRows > 0) {
-        k_prep<<<(unsigned)((P.totRows + 255) / 256), 256, 0, st>>>(P);
+        launch_next(k_prep, dim3((unsigned)((P.totRows + 255) / 256)), dim3(256), 0, st, P);
         ++*launches;
     }
     if (P.totMask > 0) {  // also writes the (zero) masks of queries without polytopes
         const long long many = member_items(P), need = (P.totMask * 32 + 255) / 256;
         if (many >= 4LL * num_sms)
-            k_member_many<<<(unsigned)(many < num_sms * 8 ? many : num_sms * 8), MEM_STATES, 0, st>>>(P);
+            launch_next(k_member_many, dim3((unsigned)(many < num_sms * 8 ? many : num_sms * 8)), dim3(MEM_STATES), 0, st, P);
         else
-            k_member<<<(unsigned)(need < num_sms * 4 ? need : num_sms * 4), 256, 0, st>>>(P);
+            launch_next(k_member, dim3((unsigned)(need < num_sms * 4 ? need : num_sms * 4)), dim3(256), 0, st, P);
         ++*launches;
     }
     if (P.totPoly > 0) {
-        k_lists<<<(unsigned)P.totPoly, 1024, 0, st>>>(P);
+        launch_next(k_lists, dim3((unsigned)P.totPoly), dim3(1024), 0, st, P);
         ++*launches;
     }
-    k_setup<<<P.Q, 1024, 0, st>>>(P);
-    k_batch<<<1, 1024, 0, st>>>(P);
+    launch_next(k_setup, dim3(P.Q), dim3(1024), 0, st, P);
+    launch_next(k_batch, dim3(1), dim3(1024), 0, st, P);
     *launches += 2;
     if (P.totN > 0 && P.totPoly > 0) {
-        k_zero_slots<<<num_sms * 8, 256, 0, st>>>(P);
+        launch_next(k_zero_slots, dim3(num_sms * 8), dim3(256), 0, st, P);
         ++*launches;
         int rc = 0;
         if (P.m == 2 && P.g == 2 && P.p == 3) rc = launch_pairs<2, 2, 3>(P, st, num_sms, ctas_per_sm, e0, e1, launches);
@@ -3930,13 +3950,13 @@ int launch_build(const BuildParams& P, void* stream, int num_sms, int ctas_per_s
         if (rc) return rc;
     }
     if (P.totN > 0) {
-        cudaMemsetAsync(P.rowCount, 0, sizeof(int) * (size_t)P.totN, st);
+        if (P.totPoly == 0) cudaMemsetAsync(P.rowCount, 0, sizeof(int) * (size_t)P.totN, st);  // else k_zero_slots clears them
         if (P.totPoly > 0) {
-            k_emit<<<num_sms * 16, 256, 0, st>>>(P);
+            launch_next(k_emit, dim3(num_sms * 16), dim3(256), 0, st, P);
             ++*launches;
         }
     }
-    k_scan<<<P.Q, 1024, 0, st>>>(P);
+    launch_next(k_scan, dim3(P.Q), dim3(1024), 0, st, P);
     ++*launches;
     if (P.totN > 0 && P.totPoly > 0) {
         // staged ids and slot indices per warp (a row holds fewer than N
@@ -3947,7 +3967,7 @@ int launch_build(const BuildParams& P, void* stream, int num_sms, int ctas_per_s
         const size_t smem = ((size_t)8 * run_cap * sizeof(int) + 1023) & ~(size_t)1023;
         const cudaError_t ea = cudaFuncSetAttribute(k_compact_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (ea != cudaSuccess) return (int)ea;
-        k_compact_fill<<<num_sms * 4, 256, smem, st>>>(P, run_cap);
+        launch_next(k_compact_fill, dim3(num_sms * 4), dim3(256), smem, st, P, run_cap);
         ++*launches;
         if (P.cost64) {
             int rc = 0;

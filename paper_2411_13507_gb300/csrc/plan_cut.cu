@@ -365,6 +365,7 @@ CDEV void obstacle_boxes(const CutParams& C, long long gw, long long nw) {
 // ---------------------------------------------------------------------------
 template <int M>
 __global__ void __launch_bounds__(256) k_cut_prep(CutParams C, int row_blocks, int copy_blocks) {
+    after_stream<false>();
     if ((int)blockIdx.x >= row_blocks + copy_blocks) {  // certified boxes, one warp per obstacle
         const long long gw = ((long long)(blockIdx.x - row_blocks - copy_blocks) * blockDim.x + threadIdx.x) >> 5;
         const long long nw = ((long long)(gridDim.x - row_blocks - copy_blocks) * blockDim.x) >> 5;
@@ -445,6 +446,7 @@ CDEV void flush_pairs(const CutParams& C, unsigned long long* buf, int n, int la
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(256) k_cut_scan(CutParams C, int target_items) {
+    after_stream<false>();
     constexpr int NP = PD + 1, BW = M == 2 ? 1 : 2;  // float4 per staged box
     constexpr int TILE = SCAN_TILE / BW;  // a multiple of SCAN_STEP
     __shared__ float4 sbox[TILE * BW];
@@ -963,6 +965,7 @@ CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, b
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD, int RB>
 __global__ void __launch_bounds__(128) k_cut_pair(CutParams C) {
+    after_stream<false>();
     constexpr int NP = PD + 1;
     static_assert(NP + RB <= 32, "lambda and y fit one warp-sized buffer");
     __shared__ float s_mix[4][32];
@@ -1141,6 +1144,7 @@ CDEV int block_excl_scan(int v, int& total) {
 }
 
 __global__ void __launch_bounds__(FILL_THREADS) k_cut_count(CutParams C) {
+    after_stream<true>();
     const long long E = block_edges(C);
     const long long nch = (E + CUT_CHUNK - 1) / CUT_CHUNK;
     for (long long c = blockIdx.x; c < nch; c += gridDim.x) {
@@ -1157,6 +1161,7 @@ __global__ void __launch_bounds__(FILL_THREADS) k_cut_count(CutParams C) {
 // One block: exclusive prefix of the chunk counts, the output count, the
 // capacity checks (output and both game lists).
 __global__ void __launch_bounds__(1024) k_cut_offsets(CutParams C) {
+    after_stream<true>();
     const long long E = block_edges(C);
     const long long nch = (E + CUT_CHUNK - 1) / CUT_CHUNK;
     __shared__ long long s_w[32];
@@ -1226,6 +1231,7 @@ CDEV double edge_cost64(const CutParams& C, const double* xi, const double* xj, 
 
 template <int M, int G, int PD>
 __global__ void __launch_bounds__(FILL_THREADS) k_cut_fill(CutParams C) {
+    after_stream<false>();
     constexpr int N_ = M * G;
     const long long E = block_edges(C);
     const long long nch = (E + CUT_CHUNK - 1) / CUT_CHUNK;
@@ -1289,6 +1295,7 @@ __global__ void __launch_bounds__(FILL_THREADS) k_cut_fill(CutParams C) {
 
 // Row offsets of the output: the output index of each row's first input edge.
 __global__ void k_cut_rows(CutParams C) {
+    after_stream<true>();
     const long long E = block_edges(C);
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > C.N || cut_failed(C.info)) return;
@@ -1304,20 +1311,20 @@ int launch_cut_t(const CutParams& C, cudaStream_t st, int num_sms, int* launches
     const long long orows = (long long)C.n_obst * C.max_orows;
     const int obst_blocks = (int)((orows + 255) / 256);
     const int box_blocks = (C.n_obst + 7) / 8;
-    k_cut_prep<M><<<row_blocks + obst_blocks + box_blocks, 256, 0, st>>>(C, row_blocks, obst_blocks);
+    launch_next(k_cut_prep<M>, dim3(row_blocks + obst_blocks + box_blocks), dim3(256), 0, st, C, row_blocks, obst_blocks);
     // pass A: a grid-stride loop over (256-unit group, obstacle stripe) items
     const int ga = num_sms * 8;
     if (e0) cudaEventRecord(e0, st);
-    k_cut_scan<M, G, PD><<<ga, 256, 0, st>>>(C, num_sms * 6);
+    launch_next(k_cut_scan<M, G, PD>, dim3(ga), dim3(256), 0, st, C, num_sms * 6);
     if (e1) cudaEventRecord(e1, st);
-    if (C.max_orows <= 8) k_cut_pair<M, G, PD, 8><<<num_sms * 4, 128, 0, st>>>(C);
-    else k_cut_pair<M, G, PD, CUT_RMAX><<<num_sms * 4, 128, 0, st>>>(C);
+    if (C.max_orows <= 8) launch_next(k_cut_pair<M, G, PD, 8>, dim3(num_sms * 4), dim3(128), 0, st, C);
+    else launch_next(k_cut_pair<M, G, PD, CUT_RMAX>, dim3(num_sms * 4), dim3(128), 0, st, C);
     long long gc = C.nchunks < (long long)num_sms * 4 ? C.nchunks : (long long)num_sms * 4;
     if (gc < 1) gc = 1;
-    k_cut_count<<<(int)gc, FILL_THREADS, 0, st>>>(C);
-    k_cut_offsets<<<1, 1024, 0, st>>>(C);
-    k_cut_fill<M, G, PD><<<(int)gc, FILL_THREADS, 0, st>>>(C);
-    k_cut_rows<<<(int)((C.N + 1 + 255) / 256), 256, 0, st>>>(C);
+    launch_next(k_cut_count, dim3((int)gc), dim3(FILL_THREADS), 0, st, C);
+    launch_next(k_cut_offsets, dim3(1), dim3(1024), 0, st, C);
+    launch_next(k_cut_fill<M, G, PD>, dim3((int)gc), dim3(FILL_THREADS), 0, st, C);
+    launch_next(k_cut_rows, dim3((int)((C.N + 1 + 255) / 256)), dim3(256), 0, st, C);
     *launches += 7;
     return (int)cudaGetLastError();
 }

@@ -399,4 +399,41 @@ int launch_refine(const RefineParams& R, void* stream, int* launches);
 int launch_cut(const CutParams& C, void* stream, int num_sms, int* launches, void* ev_scan_begin, void* ev_scan_end);
 int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launches);
 
+#ifdef __CUDACC__
+// Kernels of one call follow one another in the stream and each needs the one
+// before it whole, but a kernel of a few microseconds spends as long again
+// being launched and drained.  launch_next lets a kernel be set up while the
+// one before still runs (programmatic dependent launch); after_stream, the
+// first statement of such a kernel, waits until every earlier kernel has
+// finished and its stores are visible.  Every block must call it before it
+// reads, writes or returns: a kernel then never finishes before the ones it
+// follows, so waiting for the kernel before is waiting for them all.
+//
+// short_one: the kernel fills only a part of the GPU for a few microseconds, so
+// the next one's blocks may take the free places at once.  The others let them
+// in as their own blocks leave: next to a full GPU the blocks of the next
+// kernel would crowd onto the SMs that empty first (k_cost64 behind k_halves64:
+// its edges on few FP64 units, 5 us lost in 170).
+template <bool short_one>
+__device__ __forceinline__ void after_stream() {
+    if (short_one) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+#endif
+
 }  // namespace plan

@@ -43,6 +43,7 @@ PDEV float pld32(const void* p, long long i, int f32) {
 // Obstacle rows as {A_0, A_1, A_2, b} (FP32, for the inside test), max_orows
 // per obstacle, with row-count checks.
 __global__ void k_planes_prep(PlanesParams Q) {
+    after_stream<true>();
     const long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= (long long)Q.n_obst * Q.max_orows) return;
     const int o = (int)(u / Q.max_orows), k = (int)(u % Q.max_orows);
@@ -130,6 +131,7 @@ PDEV void unit_row(const PlanesParams& Q, int r0, int r, double* n, double& c) {
 // edge's own unit normal and offset, in 3-D the unit normals of its two
 // facets.
 __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
+    after_stream<true>();
     constexpr int M = 3;
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -235,6 +237,7 @@ PDEV float turn(float ax, float ay, float nx, float ny) {
 // so what counts is their number a lane: divisions by 2 rows instead of 7,
 // one root instead of three (500 obstacles: 2.6 + 19 -> 12 us).
 __global__ void __launch_bounds__(128) k_planes_geom2(PlanesParams Q) {
+    after_stream<true>();
     const int lane = threadIdx.x & 31, rs = lane & 3;
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -357,6 +360,7 @@ PDEV float pdot(const float4& f, const float* z) {
 // of every obstacle, min-reduced (non-negative floats order as their bits).
 template <int M>
 __global__ void __launch_bounds__(256) k_planes_ub(PlanesParams Q) {
+    after_stream<false>();
     const long long total = (long long)Q.P * Q.n_obst;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -581,6 +585,7 @@ PDEV void pair_closest(const float (&v)[M], const Geom<SH>& geo, float (&z)[M], 
 // 64-bit key (distance bits << 32 | obstacle), min-reduced per warp first.
 template <int M>
 __global__ void __launch_bounds__(256) k_planes(PlanesParams Q) {
+    after_stream<false>();
     __shared__ int s_fail;
     if (threadIdx.x == 0) s_fail = p_failed(Q.info);
     __syncthreads();
@@ -687,6 +692,7 @@ __global__ void __launch_bounds__(256) k_planes(PlanesParams Q) {
 constexpr int PL_THREADS = 384, PL_NP = 4;
 
 __global__ void __launch_bounds__(PL_THREADS, 2) k_planes_all(PlanesParams Q, int ob, int chunk) {
+    after_stream<false>();
     extern __shared__ float4 geo_sm[];
     __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, stride = ob + 1, n4 = Q.max_orows + EDGE_F4 * Q.max_edges;
@@ -773,6 +779,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_planes_all(PlanesParams Q, in
 }
 
 __global__ void k_planes_nearest(PlanesParams Q) {
+    after_stream<true>();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= Q.P || p_failed(Q.info)) return;
     const unsigned long long key = Q.keys[p];
@@ -788,10 +795,10 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
     const long long orows = (long long)Q.n_obst * Q.max_orows;
     if (orows > 0) {
         if (Q.m == 2) {
-            k_planes_geom2<<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
+            launch_next(k_planes_geom2, dim3((Q.n_obst + 3) / 4), dim3(128), 0, st, Q);
         } else {
-            k_planes_prep<<<(int)((orows + 255) / 256), 256, 0, st>>>(Q);
-            k_planes_geom<<<(Q.n_obst + 3) / 4, 128, 0, st>>>(Q);
+            launch_next(k_planes_prep, dim3((int)((orows + 255) / 256)), dim3(256), 0, st, Q);
+            launch_next(k_planes_geom, dim3((Q.n_obst + 3) / 4), dim3(128), 0, st, Q);
             ++*launches;
         }
         ++*launches;
@@ -801,8 +808,8 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
         long long grid = (total + 255) / 256;
         if (grid > (long long)num_sms * 16) grid = (long long)num_sms * 16;
         if (Q.ub) {
-            if (Q.m == 2) k_planes_ub<2><<<(int)grid, 256, 0, st>>>(Q);
-            else k_planes_ub<3><<<(int)grid, 256, 0, st>>>(Q);
+            if (Q.m == 2) launch_next(k_planes_ub<2>, dim3((int)grid), dim3(256), 0, st, Q);
+            else launch_next(k_planes_ub<3>, dim3((int)grid), dim3(256), 0, st, Q);
             ++*launches;
         }
         // all pairs in 2-D: obstacles in blocks of whole warps, and as many
@@ -820,16 +827,16 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
             if (chunks > most) chunks = most;
             if (chunks > 65535) chunks = 65535;
             const int chunk = (int)((Q.P + chunks - 1) / chunks);
-            k_planes_all<<<dim3((unsigned)nb, (unsigned)((Q.P + chunk - 1) / chunk)), PL_THREADS, smem, st>>>(Q, ob, chunk);
+            launch_next(k_planes_all, dim3((unsigned)nb, (unsigned)((Q.P + chunk - 1) / chunk)), dim3(PL_THREADS), smem, st, Q, ob, chunk);
         } else if (Q.m == 2) {
-            k_planes<2><<<(int)grid, 256, 0, st>>>(Q);
+            launch_next(k_planes<2>, dim3((int)grid), dim3(256), 0, st, Q);
         } else {
-            k_planes<3><<<(int)grid, 256, 0, st>>>(Q);
+            launch_next(k_planes<3>, dim3((int)grid), dim3(256), 0, st, Q);
         }
         ++*launches;
     }
     if (Q.P > 0 && (Q.nearest || Q.nearest_dist)) {
-        k_planes_nearest<<<(int)((Q.P + 255) / 256), 256, 0, st>>>(Q);
+        launch_next(k_planes_nearest, dim3((int)((Q.P + 255) / 256)), dim3(256), 0, st, Q);
         ++*launches;
     }
     if (Q.P > 0 && Q.nearest_plane && Q.nearest) {
@@ -846,8 +853,8 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
         Q2.nearest_dist = nullptr;
         long long grid = (Q.P + 255) / 256;
         if (grid > (long long)num_sms * 16) grid = (long long)num_sms * 16;
-        if (Q.m == 2) k_planes<2><<<(int)grid, 256, 0, st>>>(Q2);
-        else k_planes<3><<<(int)grid, 256, 0, st>>>(Q2);
+        if (Q.m == 2) launch_next(k_planes<2>, dim3((int)grid), dim3(256), 0, st, Q2);
+        else launch_next(k_planes<3>, dim3((int)grid), dim3(256), 0, st, Q2);
         ++*launches;
     }
     return (int)cudaGetLastError();
