@@ -964,7 +964,7 @@ CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, b
 // shared memory.
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD, int RB>
-__global__ void __launch_bounds__(128) k_cut_pair(CutParams C) {
+__global__ void __launch_bounds__(128, RB <= 8 && M == 2 ? 4 : 1) k_cut_pair(CutParams C) {
     after_stream<false>();
     constexpr int NP = PD + 1;
     static_assert(NP + RB <= 32, "lambda and y fit one warp-sized buffer");
