@@ -727,14 +727,49 @@ CDEV double half64(const double* coef, const double* x, int stride) {
 // game's mixes (mix: lambda then y) as certificates, then the game itself with
 // the warp as the tableau (lane r = basic row r) and exact-rounding
 // certificates; a game certified neither way is a tie (|delta*| at rounding
-// level), decided by the sign of its computed value.  GB300's FP64 pipe is
-// narrow, so the FP64 instruction count stays low: the coordinates are
-// computed once per warp, not once per lane, and the reciprocals come from an
-// FP32 estimate and two Newton steps.  Returns 1 (hit) or -1 (miss).
+// level), decided by the sign of its computed value.  Returns 1 (hit) or -1
+// (miss).
+//
+// One entry is a serial chain on a narrow FP64 pipe and ends the kernel, so the
+// FP64 instruction count stays low: coordinates once per warp, not once per
+// lane; reciprocals from an FP32 estimate and two Newton steps, one per pivot;
+// comparisons and warp minima on integer keys; the objective row as a row of
+// the tableau (lane 31) instead of a copy in every lane; certificate sums by
+// control point instead of warp reductions.  64,129 entries, 43,405 games, 26 of
+// them settled here: k_cut_pair 47 -> 36 us.
 // ---------------------------------------------------------------------------
-CDEV double warp_sum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+// Key of a double whose unsigned order is the double's order (no NaN), so that
+// comparisons and warp minima run on the integer pipe.
+CDEV unsigned long long order_key(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return b ^ ((unsigned long long)((long long)b >> 63) | 0x8000000000000000ull);
+}
+CDEV double key_value(unsigned long long k) {
+    return __longlong_as_double((long long)(k ^ (k >> 63 ? 0x8000000000000000ull : ~0ull)));
+}
+constexpr unsigned long long KEY_INF = 0xFFF0000000000000ull;  // order_key(+inf)
+
+// Warp minimum of the keys.
+CDEV unsigned long long warp_min(unsigned long long k) {
+    const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(k >> 32));
+    const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0xffffffffu);
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// The miss certificate on the canonical margins (s_g[r][l], nr facets, weights
+// s_y[r]): sum_r y_r g > km sum_r y_r |g| for every l.  Lane l takes control
+// point l: 2 nr FP64 instructions in place of a warp reduction per l and sum.
+template <int NP>
+CDEV bool miss_certified(const double* s_g, const double* s_y, int nr) {
+    const int l = (threadIdx.x & 31) < NP ? threadIdx.x & 31 : 0;
+    double ks = 0.0, ka = 0.0;
+    for (int r = 0; r < nr; ++r) {
+        const double g = s_g[r * NP + l], y = s_y[r];
+        ks = fma(y, g, ks);
+        ka = fma(y, fabs(g), ka);
+    }
+    const double km = 2.0 * (32 + 2) * U64;
+    return __all_sync(0xffffffffu, ks - km * ka > 0.0);
 }
 
 // 1 / x for the pivots (|x| within FP32 range): FP32 estimate, two Newton
@@ -749,7 +784,7 @@ CDEV double rcp64(double x) {
 }
 
 template <int M, int G, int PD>
-CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, bool& tie) {
+CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, double* s_g, double* s_y, bool& tie) {
     constexpr int N_ = M * G, NP = PD + 1, TG = 2 * G;
     static_assert(NP * M <= 32, "one control-point coordinate per lane");
     const int lane = threadIdx.x & 31;
@@ -804,146 +839,126 @@ CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, b
         for (int l = 0; l < NP; ++l) out = out && g[l] > 0.0;
         if (__ballot_sync(0xffffffffu, out) != 0u) verdict = -1;
     }
-    if (verdict == 0 && mix) {  // the FP32 game's mixes on the canonical margins
-        double L = 0.0, s = 0.0, a = 0.0;
+    if (verdict != 0) return verdict;
+    if (mine) {
+#pragma unroll
+        for (int l = 0; l < NP; ++l) s_g[lane * NP + l] = g[l];
+        s_y[lane] = (double)mix[NP + lane];
+    }
+    __syncwarp();
+    const double kh = 2.0 * (NP + 2) * U64;
+    {  // the FP32 game's mixes on the canonical margins
+        double L = 0.0, sm = 0.0, am = 0.0;
 #pragma unroll
         for (int l = 0; l < NP; ++l) {
             const double lm = (double)mix[l];
             L += lm;
-            s += lm * g[l];
-            a += lm * fabs(g[l]);
+            sm += lm * g[l];
+            am += lm * fabs(g[l]);
         }
-        const double kh = 2.0 * (NP + 2) * U64, km = 2.0 * (32 + 2) * U64;
-        if (L > 0.0 && __ballot_sync(0xffffffffu, mine && !(s + kh * a < 0.0)) == 0u) verdict = 1;
-        if (verdict == 0) {
-            const double yr = mine ? (double)mix[NP + lane] : 0.0;
-            bool miss_ok = true;
-#pragma unroll
-            for (int l = 0; l < NP; ++l) {
-                const double ks = warp_sum(yr * g[l]), ka = warp_sum(yr * fabs(g[l]));
-                miss_ok = miss_ok && (ks - km * ka > 0.0);
-            }
-            if (miss_ok) verdict = -1;
-        }
+        if (L > 0.0 && __ballot_sync(0xffffffffu, mine && !(sm + kh * am < 0.0)) == 0u) return 1;
+        if (miss_certified<NP>(s_g, s_y, nr)) return -1;
     }
-        if (verdict == 0) {
-            double gmin = inf;
+    unsigned long long kmin = ~0ull;
 #pragma unroll
-            for (int l = 0; l < NP; ++l) gmin = mine ? fmin(gmin, g[l]) : gmin;
-            for (int of = 16; of > 0; of >>= 1) gmin = fmin(gmin, __shfl_xor_sync(0xffffffffu, gmin, of));
-            const double shift = 1.0 - gmin;
-            double T[NP], rhs = mine ? 1.0 : 0.0, d[NP];
-            int colLab[NP], rowLab = NP + lane;
+    for (int l = 0; l < NP; ++l) {
+        const unsigned long long k = mine ? order_key(g[l]) : ~0ull;
+        kmin = k < kmin ? k : kmin;
+    }
+    const double shift = 1.0 - key_value(warp_min(kmin));
+    // lane r < nr: basic row r; lane 31 (never a facet's): the objective row d
+    const bool obj = lane == 31;
+    double T[NP], rhs = mine ? 1.0 : 0.0;
+    int colLab[NP], rowLab = NP + lane;
 #pragma unroll
-            for (int l = 0; l < NP; ++l) {
-                T[l] = mine ? g[l] + shift : 0.0;
-                d[l] = 1.0;
-                colLab[l] = l;
-            }
-            const double tol = 1e-13;
-            for (int it = 0; it < GAME_ITERS; ++it) {
-                int c = -1, cl = 1 << 20;
-                double dbest = tol;
-                if (it < GAME_DANTZIG) {
-#pragma unroll
-                    for (int l = 0; l < NP; ++l)
-                        if (d[l] > dbest) {
-                            c = l;
-                            dbest = d[l];
-                        }
-                    if (c >= 0) {
-#pragma unroll
-                        for (int l = 0; l < NP; ++l) cl = (l == c) ? colLab[l] : cl;
-                    }
-                } else {
-#pragma unroll
-                    for (int l = 0; l < NP; ++l)
-                        if (d[l] > tol && colLab[l] < cl) {
-                            c = l;
-                            cl = colLab[l];
-                        }
-                }
-                if (c < 0) break;
-                double colc = T[0];
-#pragma unroll
-                for (int l = 1; l < NP; ++l) colc = (l == c) ? T[l] : colc;
-                const bool ok = mine && colc > tol;
-                double best = ok ? rhs * rcp64(colc) : inf;
-                int bl = ok ? rowLab : (1 << 20), bi = lane;
-                for (int of = 16; of > 0; of >>= 1) {
-                    const double ob = __shfl_xor_sync(0xffffffffu, best, of);
-                    const int obl = __shfl_xor_sync(0xffffffffu, bl, of);
-                    const int obi = __shfl_xor_sync(0xffffffffu, bi, of);
-                    if (ob < best || (ob == best && obl < bl)) {
-                        best = ob;
-                        bl = obl;
-                        bi = obi;
-                    }
-                }
-                if (!(best < inf)) break;  // unbounded: impossible with payoffs >= 1
-                const int r = bi;
-                const double p = __shfl_sync(0xffffffffu, colc, r);
-                const double inv = rcp64(p);
-                double rs[NP];
-#pragma unroll
-                for (int l = 0; l < NP; ++l) {
-                    const double v = __shfl_sync(0xffffffffu, T[l], r);
-                    rs[l] = (l == c) ? inv : v * inv;
-                }
-                const double rhs_s = __shfl_sync(0xffffffffu, rhs, r) * inv;
-                const int lr = __shfl_sync(0xffffffffu, rowLab, r);
-                if (lane == r) {
-#pragma unroll
-                    for (int l = 0; l < NP; ++l) T[l] = rs[l];
-                    rhs = rhs_s;
-                    rowLab = cl;
-                } else {
-#pragma unroll
-                    for (int l = 0; l < NP; ++l) T[l] = ((l == c) ? 0.0 : T[l]) - colc * rs[l];
-                    rhs = rhs - colc * rhs_s;
-                }
-                double dc = d[0];
-#pragma unroll
-                for (int l = 1; l < NP; ++l) dc = (l == c) ? d[l] : dc;
-#pragma unroll
-                for (int l = 0; l < NP; ++l) {
-                    d[l] = ((l == c) ? 0.0 : d[l]) - dc * rs[l];
-                    colLab[l] = (l == c) ? lr : colLab[l];
-                }
-            }
-            double lam[NP], L = 0.0;
+    for (int l = 0; l < NP; ++l) {
+        T[l] = mine ? g[l] + shift : (obj ? 1.0 : 0.0);
+        colLab[l] = l;
+    }
+    const double tol = 1e-13;
+    const unsigned long long ktol = order_key(tol);
+    for (int it = 0; it < GAME_ITERS; ++it) {
+        int c = -1;  // of the objective row's lane
+        if (it < GAME_DANTZIG) {
+            unsigned long long dbest = ktol;
 #pragma unroll
             for (int l = 0; l < NP; ++l) {
-                lam[l] = warp_sum(rowLab == l ? pos_part(rhs) : 0.0);
-                L += lam[l];
+                const unsigned long long k = order_key(T[l]);
+                if (k > dbest && k <= KEY_INF) {
+                    c = l;
+                    dbest = k;
+                }
             }
-            double yr = 0.0;  // this lane's facet weight
-#pragma unroll
-            for (int l = 0; l < NP; ++l)
-                if (colLab[l] == NP + lane) yr = pos_part(-d[l]);
-            if (!mine) yr = 0.0;
-            const double kh = 2.0 * (NP + 2) * U64, km = 2.0 * (32 + 2) * U64;
-            double s = 0.0, a = 0.0;
+        } else {
+            int cb = 1 << 20;
 #pragma unroll
             for (int l = 0; l < NP; ++l) {
-                s += lam[l] * g[l];
-                a += lam[l] * fabs(g[l]);
-            }
-            const bool hit_ok = L > 0.0 && __ballot_sync(0xffffffffu, mine && !(s + kh * a < 0.0)) == 0u;
-            bool miss_ok = true;
-#pragma unroll
-            for (int l = 0; l < NP; ++l) {
-                const double ks = warp_sum(yr * g[l]), ka = warp_sum(yr * fabs(g[l]));
-                miss_ok = miss_ok && (ks - km * ka > 0.0);
-            }
-            if (hit_ok) verdict = 1;
-            else if (miss_ok) verdict = -1;
-            else {
-                verdict = (L > 0.0 && 1.0 / L - shift <= 0.0) ? 1 : -1;
-                tie = true;
+                const unsigned long long k = order_key(T[l]);
+                if (k > ktol && k <= KEY_INF && colLab[l] < cb) {
+                    c = l;
+                    cb = colLab[l];
+                }
             }
         }
-    return verdict;
+        c = __shfl_sync(0xffffffffu, c, 31);
+        if (c < 0) break;
+        int cl = colLab[0];
+        double colc = T[0];
+#pragma unroll
+        for (int l = 1; l < NP; ++l) {
+            colc = (l == c) ? T[l] : colc;
+            cl = (l == c) ? colLab[l] : cl;
+        }
+        const bool ok = mine && colc > tol;
+        const double rc = rcp64(colc);
+        // least ratio, ties to the least label; + 0.0 so that -0 ties with 0
+        const unsigned long long ratio = ok ? order_key(fma(rhs, rc, 0.0)) : ~0ull;
+        const unsigned long long best = warp_min(ratio);
+        if (best >= KEY_INF) break;  // unbounded: impossible with payoffs >= 1
+        const int r = (int)(__reduce_min_sync(0xffffffffu, ratio == best ? (unsigned)(rowLab << 5 | lane) : 0xffffffffu) & 31u);
+        const double inv = __shfl_sync(0xffffffffu, rc, r);
+        double rs[NP];
+#pragma unroll
+        for (int l = 0; l < NP; ++l) {
+            const double v = __shfl_sync(0xffffffffu, T[l], r);
+            rs[l] = (l == c) ? inv : v * inv;
+        }
+        const double rhs_s = __shfl_sync(0xffffffffu, rhs, r) * inv;
+        const int lr = __shfl_sync(0xffffffffu, rowLab, r);
+        if (lane == r) {
+#pragma unroll
+            for (int l = 0; l < NP; ++l) T[l] = rs[l];
+            rhs = rhs_s;
+            rowLab = cl;
+        } else {
+#pragma unroll
+            for (int l = 0; l < NP; ++l) T[l] = ((l == c) ? 0.0 : T[l]) - colc * rs[l];
+            rhs = rhs - colc * rhs_s;
+        }
+#pragma unroll
+        for (int l = 0; l < NP; ++l) colLab[l] = (l == c) ? lr : colLab[l];
+    }
+    double L = 0.0, sm = 0.0, am = 0.0, yr = 0.0;  // yr: this lane's facet weight
+    const double rp = pos_part(rhs);
+#pragma unroll
+    for (int l = 0; l < NP; ++l) {
+        const unsigned at = __ballot_sync(0xffffffffu, rowLab == l);
+        const double v = __shfl_sync(0xffffffffu, rp, at ? __ffs(at) - 1 : 0);
+        const double lam = at ? v : 0.0;
+        L += lam;
+        sm += lam * g[l];
+        am += lam * fabs(g[l]);
+        const double d = __shfl_sync(0xffffffffu, T[l], 31);
+        if (colLab[l] == NP + lane) yr = pos_part(-d);
+    }
+    __syncwarp();  // the mix's weights are read
+    if (mine) s_y[lane] = yr;
+    __syncwarp();
+    const bool hit_ok = L > 0.0 && __ballot_sync(0xffffffffu, mine && !(sm + kh * am < 0.0)) == 0u;
+    if (hit_ok) return 1;
+    if (miss_certified<NP>(s_g, s_y, nr)) return -1;
+    tie = true;
+    return (L > 0.0 && 1.0 / L - shift <= 0.0) ? 1 : -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -959,34 +974,35 @@ CDEV int settle64(const CutParams& C, unsigned long long en, const float* mix, b
 //   miss: y >= 0 and for every l
 //         sum_r y_r G[l][r] - sum_r y_r band_r - 2 (RB + 2) u sum_r y_r |G[l][r]| > 0.
 // The margins are recomputed for the checks rather than kept in registers.
-// Entries no FP32 certificate settles are then settled one by one by the
-// whole warp in FP64 (settle64), with the lane's lambda and y passed through
-// shared memory.
+// Entries no FP32 certificate settles are then settled in FP64 by a warp each
+// (settle64), shared out over the block's warps: neighbours in the list tend to
+// be near the same obstacle, so one warp of a block often has several (36 -> 34
+// us on the entries above).
 // ---------------------------------------------------------------------------
 template <int M, int G, int PD, int RB>
 __global__ void __launch_bounds__(128, RB <= 8 && M == 2 ? 4 : 1) k_cut_pair(CutParams C) {
     after_stream<false>();
     constexpr int NP = PD + 1;
-    static_assert(NP + RB <= 32, "lambda and y fit one warp-sized buffer");
-    __shared__ float s_mix[4][32];
+    static_assert(RB < 31, "the objective row has a lane of its own");
+    __shared__ float s_mix[128][NP + RB];            // entries to settle: lambda, then y
+    __shared__ unsigned long long s_todo[128];
+    __shared__ int s_n;
+    __shared__ double s_g[4][RB * NP], s_y[4][RB];
     const long long n = block_count(C.info, &C.info->cut_near, C.cap32);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     unsigned long long n_s1 = 0, n_s2 = 0, n_games = 0, n_64 = 0, n_ties = 0;
-    for (long long k0 = gw * 32; k0 < n; k0 += nw * 32) {
-        const long long k = k0 + lane;
+    for (long long k0 = (long long)blockIdx.x * 128; k0 < n; k0 += (long long)gridDim.x * 128) {
+        const long long k = k0 + threadIdx.x;
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
         unsigned long long en = 0;
-        bool need64 = false;
         float lam[NP], y[RB];
-        long long e = 0;
-        int t = 0;
         if (k < n) {
             en = C.list32[k];
             const long long u = (long long)(en >> OBST_BITS);
             const int o = (int)(en & ((1ull << OBST_BITS) - 1ull));
-            e = u / C.nT;
-            t = (int)(u - e * C.nT);
+            const long long e = u / C.nT;
+            const int t = (int)(u - e * C.nT);
             if (!((*(volatile const uint32_t*)(C.hit + e) >> t) & 1u)) {
                 float P[NP * M], S, lo[M], hi[M];
                 unit_points<M, G, PD>(C, C.src[e], C.col_in[e], t, P, S, lo, hi);
@@ -1071,33 +1087,31 @@ __global__ void __launch_bounds__(128, RB <= 8 && M == 2 ? 4 : 1) k_cut_pair(Cut
                     for (int l = 0; l < NP; ++l) miss_ok = miss_ok && (ks[l] - Y - km * ka[l] > 0.f);
                     if (hit_ok) atomicOr(&C.hit[e], 1u << t);
                     else if (!miss_ok) {
-                        need64 = true;
+                        const int q = atomicAdd(&s_n, 1);
+                        s_todo[q] = en;
 #pragma unroll
-                        for (int r = 0; r < RB; ++r) y[r] = r < nr ? y[r] : 0.f;
+                        for (int l = 0; l < NP; ++l) s_mix[q][l] = lam[l];
+#pragma unroll
+                        for (int r = 0; r < RB; ++r) s_mix[q][NP + r] = r < nr ? y[r] : 0.f;
                     }
                 }
             }
         }
-        // entries no FP32 certificate settled: the whole warp, one at a time
-        for (unsigned todo = __ballot_sync(0xffffffffu, need64); todo; todo &= todo - 1u) {
-            const int src = __ffs(todo) - 1;
-            if (lane == src) {
-#pragma unroll
-                for (int l = 0; l < NP; ++l) s_mix[warp][l] = lam[l];
-#pragma unroll
-                for (int r = 0; r < RB; ++r) s_mix[warp][NP + r] = y[r];
-            }
-            __syncwarp();
-            const unsigned long long en_s = __shfl_sync(0xffffffffu, en, src);
+        // entries no FP32 certificate settled: a warp each, over the block's warps
+        __syncthreads();
+        for (int q = warp; q < s_n; q += 4) {
             bool tie;
-            const int v = settle64<M, G, PD>(C, en_s, s_mix[warp], tie);
-            if (lane == src) {
+            const unsigned long long ens = s_todo[q];
+            const int v = settle64<M, G, PD>(C, ens, s_mix[q], s_g[warp], s_y[warp], tie);
+            if (lane == 0) {
                 ++n_64;
                 n_ties += tie;
-                if (v == 1) atomicOr(&C.hit[e], 1u << t);
+                const long long u = (long long)(ens >> OBST_BITS), es = u / C.nT;
+                if (v == 1) atomicOr(&C.hit[es], 1u << (int)(u - es * C.nT));
             }
             __syncwarp();
         }
+        __syncthreads();
     }
     cut_block_add(&C.info->cut_step1, n_s1);
     cut_block_add(&C.info->cut_step2, n_s2);
