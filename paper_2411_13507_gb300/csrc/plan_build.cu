@@ -3786,8 +3786,9 @@ size_t smem_one(const BuildParams& P) {
     return f * sizeof(float);
 }
 
-// screened FP32 kernel: transposed halves, screen rows, band and cost
-// magnitudes, states, two padded tables, A|b rows and the two pair lists
+// screened FP32 kernel: records, points, screen rows and list 1 or the cost
+// halves (sc_front), band and cost magnitudes and free maxima, states, two
+// padded tables, A|b rows and list 2
 template <int M, int G, int PD>
 size_t smem_sc(const BuildParams& P) {
     using SS = ScShape<M, G, PD>;
