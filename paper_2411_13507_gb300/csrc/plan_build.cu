@@ -3573,17 +3573,21 @@ __global__ void __launch_bounds__(256) k_halves64(BuildParams P) {
 }
 
 // Which durations of an edge's mask can be the cheapest in FP64, by their FP32
-// costs.  With S = sum of the halves' magnitudes, rounding the halves and
-// their sum errs by at most 2^-24 (2 S + cost), the norms and the sum of the
-// segments by at most 2^-24 (w + PD + 4) cost for w <= 9 rows a segment and PD
-// <= 7 segments; err = 2^-20 (S + cost) is over twice that for either term and
-// leaves far more than the FP64 key's rounding between a dropped duration and
-// the cheapest one.  A NaN or infinite cost drops nothing.
+// costs.  With S = sum of the halves' magnitudes (at least the cost, up to
+// rounding), rounding the halves and their sums errs by at most 2^-24 (2 S +
+// cost), the norms and the sum of the segments by at most 2^-24 (w + PD + 4)
+// cost for w <= 9 rows a segment and PD <= 7 segments: 23/32 of 2^-20 (S + cost)
+// together at most, and the rest is far more than the FP64 key's rounding.
+// Squares below 2^-126 lose up to 2^-150 each to underflow, 3 * 2^-75 of a norm
+// and under 2^-70 of a cost, which the absolute term covers at every scale.
+// Where a cost is not finite (an overflow, NaN) the FP32 values say nothing and
+// every duration stays.
 template <int M, int PD>
-DEVI uint32_t cheapest_bits(uint32_t bits, const float* hl, const float* hr, int DR) {
+DEVI uint32_t cheapest_bits(const uint32_t mask, const float* hl, const float* hr, int DR) {
     const int W = DR * M, E = PD * W;
-    uint32_t keep = 0;
-    float ub = __int_as_float(0x7f800000), lb = ub;  // smallest upper bound; smallest lower bound of those kept
+    const float inf = __int_as_float(0x7f800000);
+    uint32_t bits = mask, keep = 0;
+    float ub = inf, lb = inf;  // smallest upper bound; smallest lower bound of those kept
     while (bits) {
         const int t = __ffs(bits) - 1;
         bits &= bits - 1u;
@@ -3599,11 +3603,12 @@ DEVI uint32_t cheapest_bits(uint32_t bits, const float* hl, const float* hr, int
             }
             cost += sqrtf(ss);
         }
-        const float err = 9.5367431640625e-07f * (S + cost);  // 2^-20
+        if (!(cost < inf)) return mask;
+        const float err = fmaf(9.5367431640625e-07f, S + cost, 1.6940658945086007e-21f);  // 2^-20 (S + cost) + 2^-69
         if (cost - err > ub) continue;
         if (cost + err < lb) {  // cheaper than every one kept so far
             keep = 0;
-            lb = __int_as_float(0x7f800000);
+            lb = inf;
         }
         keep |= 1u << t;
         lb = fminf(lb, cost - err);
