@@ -29,7 +29,7 @@ namespace {
 
 // The relaxed barrier's constants: value and slope of the quadratic below delta.
 struct Barrier {
-    float delta, inv, inv2, off;  // delta, 1 / delta, 1 / delta^2, -log delta - 1/2
+    float delta, inv, off;  // delta, 1 / delta, -log delta - 1/2
 };
 
 // phi(m) and, with GRAD, phi'(m) of one margin.
@@ -37,18 +37,19 @@ template <bool GRAD>
 DEVI float phi_one(const Barrier& B, float m, float& slope) {
     const bool in = m >= B.delta;
     const float z = (m - 2.f * B.delta) * B.inv;
-    if (GRAD) slope = in ? -1.f / m : (m - 2.f * B.delta) * B.inv2;
+    if (GRAD) slope = in ? -1.f / m : z * B.inv;  // not / delta^2, which underflows first
     return in ? -logf(m) : fmaf(0.5f * z, z, B.off);
 }
 
 // phi(c - Q) + phi(c + Q) and its derivative in Q.  Both margins in the
 // logarithm share one root of work: log m1 + log m2 = log(m1 m2), and the two
-// reciprocals come from one (m1 + m2 = 2 c, so the product stays in range for
-// every bound below 2^60; a larger one takes the margins one by one).
+// reciprocals come from one.  m1 + m2 = 2 c and both are at least delta, so the
+// product lies between c delta and c^2: in range for bounds below 2^60 with
+// c delta above 2^-125; others take the margins one by one.
 template <bool GRAD>
 DEVI float phi_pair(const Barrier& B, float c, float Q, float& slope) {
     const float m1 = c - Q, m2 = c + Q;
-    if (c > 1.152921504606847e18f) {
+    if (c > 1.152921504606847e18f || c * B.delta < 2.350988701644575e-38f) {
         float s1 = 0.f, s2 = 0.f;
         const float v = phi_one<GRAD>(B, m1, s1) + phi_one<GRAD>(B, m2, s2);
         if (GRAD) slope = s2 - s1;
@@ -56,14 +57,13 @@ DEVI float phi_pair(const Barrier& B, float c, float Q, float& slope) {
     }
     const bool in1 = m1 >= B.delta, in2 = m2 >= B.delta;
     const float u1 = in1 ? m1 : 1.f, u2 = in2 ? m2 : 1.f, pr = u1 * u2;
-    const float d1 = m1 - 2.f * B.delta, d2 = m2 - 2.f * B.delta;
-    const float z1 = d1 * B.inv, z2 = d2 * B.inv;
+    const float z1 = (m1 - 2.f * B.delta) * B.inv, z2 = (m2 - 2.f * B.delta) * B.inv;
     float v = -logf(pr);
     v += in1 ? 0.f : fmaf(0.5f * z1, z1, B.off);
     v += in2 ? 0.f : fmaf(0.5f * z2, z2, B.off);
     if (GRAD) {
         const float r = 1.f / pr;
-        const float s1 = in1 ? -r * u2 : d1 * B.inv2, s2 = in2 ? -r * u1 : d2 * B.inv2;
+        const float s1 = in1 ? -r * u2 : z1 * B.inv, s2 = in2 ? -r * u1 : z2 * B.inv;
         slope = s2 - s1;
     }
     return v;
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(RF_SEGS * M) k_refine(RefineParams R) {
     const int nr = act ? min(R.nrows[s0 + q], rmax) : 0;
     __syncthreads();
     const float mu = R.mu, ws = R.w_snap, Ti = 1.f / T;
-    const Barrier B = {R.delta, 1.f / R.delta, 1.f / (R.delta * R.delta), -logf(R.delta) - 0.5f};
+    const Barrier B = {R.delta, 1.f / R.delta, -logf(R.delta) - 0.5f};
     float loss = 0.f, dT = 0.f;
     if (act) {
         // reach margins and snap energy of axis a (Theorem 1 per axis; the snap
