@@ -514,7 +514,7 @@ typedef struct {
 
 /*
  * Batched findPath: the same computation as plan_search for many queries, one
- * 1024-thread block per query (block barriers, no grid barrier).  Per-query
+ * to eight 1024-thread blocks of a cluster per query (no grid barrier).  Per-query
  * outcomes go to each query's status word; NO_PATH is not a batch error.
  * plan_prepare_search_batched uploads the descriptors (may allocate/wait);
  * plan_search_batched only launches (capturable in a CUDA graph).

@@ -487,8 +487,16 @@ __global__ void __launch_bounds__(1024, 1) k_search(SearchParams P) {
 // latency, and the largest query's is the batch's: a CTA per 1024 vertices, up
 // to 8 of a cluster, shortens it, and four groups of 32 edges are in flight at
 // once (256 queries of 512 to 16,384 vertices, 125 M edges: one CTA a query
-// and one group 6.55 ms, now 1.95 ms).  CTAs a small query does not need leave at
+// and one group 7.2 ms, now 1.63 ms).  CTAs a small query does not need leave at
 // once; barriers count the threads that have not left.
+//
+// With few vertices a warp the sweep's own steps count: a query of one CTA takes
+// block barriers (a cluster barrier also orders global memory), a warp finds its
+// frontier with one load a lane instead of one a vertex in series, and every CTA
+// has a flag of its own, so that no remote read follows the barrier (96 queries
+// of 100 to 1000 vertices: cluster barriers, serial flags and a remote flag 109
+// to 128 us, one CTA a query and one group 92 to 95, now 72; 256 of 300 to 1200:
+// 213, 165 and 143 us).
 // ---------------------------------------------------------------------------
 constexpr int SB_CLUSTER = 8, SB_VERTICES = 1024;
 
@@ -519,6 +527,10 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
     const int nc = min((int)cluster.num_blocks(), (N + SB_VERTICES - 1) / SB_VERTICES > 1 ? (N + SB_VERTICES - 1) / SB_VERTICES : 1);
     const int rank = (int)cluster.block_rank();
     if (rank >= nc) return;
+    auto sync = [&] {
+        if (nc > 1) cluster.sync();
+        else __syncthreads();
+    };
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     const int v0 = rank * (int)blockDim.x + tid, vstep = nc * (int)blockDim.x;   // this thread's vertices
     const int w0 = wid * nc + rank, wstep = nc * nw;                            // this warp's vertices
@@ -530,13 +542,12 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
     __shared__ int s_wi[2][32];
     __shared__ unsigned long long s_nd[2][SB_CLUSTER];  // rank 0's: every CTA's nearest start and goal
     __shared__ int s_id[2][SB_CLUSTER];
-    __shared__ int s_changed[3];                        // rank 0's: a CTA changed a distance, by sweep mod 3
-    __shared__ int s_bad, s_any;
+    __shared__ int s_changed[3];                        // a warp of the query changed a distance, by sweep mod 3
+    __shared__ int s_bad;
     if (tid == 0) {
         const long long E = *Q.count;
         s_bad = N < 1 || E < 0 || E > Q.cap;
         s_changed[0] = s_changed[1] = s_changed[2] = 0;
-        s_any = 0;
     }
     // initial values; the nearest vertices of start and goal (ties to the lowest id)
     unsigned long long kb[2] = {~0ull, ~0ull};
@@ -570,7 +581,7 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
             s_wi[q][wid] = ki[q];
         }
     }
-    cluster.sync();  // every CTA of the query runs: rank 0's shared memory can be written
+    sync();  // every CTA of the query runs: rank 0's shared memory can be written
     if (s_bad) {     // the same in all of them
         if (tid == 0 && rank == 0) {
             *Q.status = PLAN_ERR_INVALID_ARG;
@@ -585,7 +596,7 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
         *cluster.map_shared_rank(&s_nd[tid][rank], 0) = b;
         *cluster.map_shared_rank(&s_id[tid][rank], 0) = i;
     }
-    cluster.sync();
+    sync();
     int sg[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -600,44 +611,43 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
         dist[s] = 0ull;
         front[s] = 1;
     }
-    cluster.sync();
-    int* changed0 = cluster.map_shared_rank(&s_changed[0], 0);
+    sync();
     int cur = 0, it = 0;
     volatile unsigned long long* vdist = dist;
     for (;;) {
         // the slot of the next sweep: last read before the barrier that ended the sweep before this one
-        if (tid == 0 && rank == 0) s_changed[(it + 1) % 3] = 0;
+        if (tid == 0) s_changed[(it + 1) % 3] = 0;
         bool my_change = false;
         const unsigned long long gd = vdist[g];   // vertices not closer than the goal do not relax
-        for (int v = w0; v < N; v += wstep) {
-            if (!front[cur * N + v]) continue;
-            __syncwarp();
-            if (lane == 0) front[cur * N + v] = 0;
-            if (vdist[v] >= gd) continue;
-            const double dv = __longlong_as_double((long long)vdist[v]);
-            each_edge(Q, B.w_f64, N, v, lane, [&](const int (&u)[4], const double (&w)[4]) {
-                unsigned long long nd[4], old[4];
+        for (int vb = w0; vb < N; vb += 32 * wstep) {  // a lane a vertex
+            const int vl = vb + lane * wstep;
+            const bool on = vl < N && front[cur * N + vl];
+            if (on) front[cur * N + vl] = 0;
+            for (unsigned left = __ballot_sync(0xffffffffu, on); left; left &= left - 1u) {
+                const int v = vb + (__ffs(left) - 1) * wstep;
+                const unsigned long long dvb = vdist[v];
+                if (dvb >= gd) continue;
+                const double dv = __longlong_as_double((long long)dvb);
+                each_edge(Q, B.w_f64, N, v, lane, [&](const int (&u)[4], const double (&w)[4]) {
+                    unsigned long long nd[4], old[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    nd[c] = (unsigned long long)__double_as_longlong(__dadd_rn(dv, w[c]));
-                    old[c] = u[c] >= 0 && u[c] < N ? atomicMin(&dist[u[c]], nd[c]) : 0ull;
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (nd[c] < old[c]) {
-                        front[(cur ^ 1) * N + u[c]] = 1;
-                        my_change = true;
+                    for (int c = 0; c < 4; ++c) {
+                        nd[c] = (unsigned long long)__double_as_longlong(__dadd_rn(dv, w[c]));
+                        old[c] = u[c] >= 0 && u[c] < N ? atomicMin(&dist[u[c]], nd[c]) : 0ull;
                     }
-            });
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (nd[c] < old[c]) {
+                            front[(cur ^ 1) * N + u[c]] = 1;
+                            my_change = true;
+                        }
+                });
+            }
         }
-        if (my_change) s_any = 1;
-        __syncthreads();
-        if (tid == 0 && s_any) {
-            changed0[it % 3] = 1;
-            s_any = 0;
-        }
-        cluster.sync();
-        const int ch = changed0[it % 3];
+        // every CTA has its own flag, so that none reads another's after the barrier
+        if (__any_sync(0xffffffffu, my_change) && lane < nc) *cluster.map_shared_rank(&s_changed[it % 3], lane) = 1;
+        sync();
+        const int ch = s_changed[it % 3];
         ++it;
         if (!ch) break;
         if (it > B.max_sweeps) {
@@ -645,7 +655,6 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
                 *Q.status = PLAN_ERR_TIMEOUT;
                 *Q.path_len = 0;
             }
-            cluster.sync();  // rank 0's shared memory has been read
             return;
         }
         cur ^= 1;
@@ -668,7 +677,7 @@ __global__ void __launch_bounds__(1024) k_search_batched(BatchSearchParams B) {
                 }
             });
         }
-        cluster.sync();
+        sync();
     }
     if (tid == 0 && rank == 0) {
         const unsigned long long dg = vdist[g];
@@ -1511,7 +1520,7 @@ int launch_search_batched(const BatchSearchParams& P, void* stream, int* launche
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = C > 1 ? 1 : 0;
     ++*launches;
     return (int)cudaLaunchKernelEx(&cfg, k_search_batched, P);
 }
