@@ -460,6 +460,9 @@ enum { PLAN_MPC_OK = 0, PLAN_MPC_INFEASIBLE = 1, PLAN_MPC_ITERATION_LIMIT = 2 };
  * weights) and UNSUPPORTED (model or problem size); per-problem outcomes go
  * to status, not to plan_wait.  An SQP refinement alternates
  * plan_nearest_planes at the new nodes and plan_mpc_qp.
+ * Under stream capture the graph holds the parameters of the captured call: a
+ * table and a factor of its own (under 50 KB for every distinct parameter set
+ * captured, kept until plan_destroy), which each replay uploads and factors.
  */
 int plan_mpc_qp(plan_ctx* ctx, int B, const plan_mpc_params* prm, const double* x0, const double* ref,
                 const float* planes, double* x, double* u, double* obj, int32_t* status, int32_t* iters,
