@@ -186,7 +186,10 @@ int fail(plan_ctx* c, int code, const std::string& msg) {
     return code;
 }
 
+// A failed runtime call's status, with the runtime's record of it cleared: the
+// next call's launch check must not find it.
 int cuda_fail(plan_ctx* c, cudaError_t e, const char* where) {
+    cudaGetLastError();
     return fail(c, PLAN_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
