@@ -480,6 +480,7 @@ int plan_create(plan_ctx** out, const plan_model* model, void* cuda_stream) {
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->d_info, sizeof(DevInfo));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_info, 0, sizeof(DevInfo), c->stream);  // not every first call clears its status
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_info, sizeof(DevInfo));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->tab_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->stage_ev, cudaEventDisableTiming);
@@ -1661,8 +1662,9 @@ int plan_wait(plan_ctx* c, plan_info* info) {
     if (e != cudaSuccess) return cuda_fail(c, e, "stream sync");
     e = cudaMemcpy(c->h_info, c->d_info, sizeof(DevInfo), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(c, e, "read status");
-    // the status covers the work issued since the previous plan_wait: clear it
-    e = cudaMemset(c->d_info, 0, 2 * sizeof(int));
+    // the status covers the work issued since the previous plan_wait: clear it,
+    // before the work issued next
+    e = cudaMemsetAsync(c->d_info, 0, 2 * sizeof(int), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "clear status");
     const DevInfo& d = *c->h_info;
     if (d.status == PLAN_ERR_CAPACITY) {
