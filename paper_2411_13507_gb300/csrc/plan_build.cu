@@ -3834,7 +3834,7 @@ template <int M, int G, int PD, bool BF>
 int launch_tc(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_per_sm, cudaEvent_t e0, cudaEvent_t e1,
               int* launches) {
     const size_t sm = smem_tc<M, G, PD, BF>(P);
-    cudaFuncSetAttribute(k_pairs_tc<M, G, PD, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_shared<k_pairs_tc<M, G, PD, BF>>();
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_tc<M, G, PD, BF>, 256, sm);
     if (occ < 1) occ = 1;
@@ -3861,7 +3861,7 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
     }
     if (P.arith == PLAN_F64) {
         const size_t sm = smem_f64<M, G, PD>(P);
-        cudaFuncSetAttribute(k_pairs_f64<M, G, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_shared<k_pairs_f64<M, G, PD>>();
         int occ = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pairs_f64<M, G, PD>, 256, sm);
         if (occ < 1) occ = 1;
@@ -3871,7 +3871,7 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         ++*launches;
     } else if (P.pipeline == 1 && P.tile == TILE && smem_ws<M, G, PD>(P) <= 227 * 1024) {
         const size_t sm = smem_ws<M, G, PD>(P);
-        cudaFuncSetAttribute(k_pairs_ws<M, G, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        allow_shared<k_pairs_ws<M, G, PD>>();
         if (e0) cudaEventRecord(e0, st);
         launch_next(k_pairs_ws<M, G, PD>, dim3(num_sms), dim3(512), sm, st, P);
         if (e1) cudaEventRecord(e1, st);
@@ -3885,7 +3885,7 @@ int launch_pairs(const BuildParams& P, cudaStream_t st, int num_sms, int ctas_pe
         const size_t sm = sc ? smem_sc<M, G, PD>(P) : smem_one<M, G, PD>(P);
         int threads = (P.tile / 4) * (P.tile / 4);  // one thread per 4x4 micro-tile
         if (sc) threads = (threads + 31) & ~31;      // whole warps (warp-level list positions)
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        sc ? allow_shared<k_pairs_sc<M, G, PD>>() : allow_shared<k_pairs_fast<M, G, PD>>();
         int occ = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, sm);
         if (occ < 1) occ = 1;
@@ -3971,7 +3971,7 @@ int launch_build(const BuildParams& P, void* stream, int num_sms, int ctas_per_s
         // bound) fit on an SM
         const int run_cap = 2 * (P.maxN < 512 ? (P.maxN > 32 ? P.maxN : 32) : 512);
         const size_t smem = ((size_t)8 * run_cap * sizeof(int) + 1023) & ~(size_t)1023;
-        const cudaError_t ea = cudaFuncSetAttribute(k_compact_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t ea = allow_shared<k_compact_fill>();
         if (ea != cudaSuccess) return (int)ea;
         // four times the CTAs that fit: rows of several polytopes take several
         // times as long, and the scheduler evens them out where a warp's fixed

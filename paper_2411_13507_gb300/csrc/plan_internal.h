@@ -1,6 +1,7 @@
 // Internal definitions shared by the CUDA translation units of libplan.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 
 #include <vector_types.h>
@@ -418,6 +419,22 @@ template <bool short_one>
 __device__ __forceinline__ void after_stream() {
     if (short_one) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Lets KERN's launches take as much dynamic shared memory as a block can have
+// beside the kernel's static part.  The limit belongs to the kernel, not to a
+// launch: set to each launch's own size, another thread's smaller size could
+// come between setting and launching and fail the launch.
+template <auto KERN>
+inline cudaError_t allow_shared() {
+    static std::atomic<int> most{-1};  // the same for every thread and device
+    if (most < 0) {
+        cudaFuncAttributes a = {};
+        const cudaError_t e = cudaFuncGetAttributes(&a, KERN);
+        if (e != cudaSuccess) return e;
+        most = 227 * 1024 - (int)a.sharedSizeBytes;
+    }
+    return cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 template <typename... P, typename... A>

@@ -743,12 +743,12 @@ int launch_mpc(const MpcParams& P, void* stream, int* launches) {
     cudaStream_t st = (cudaStream_t)stream;
     if (!P.j0_ready) {
         const size_t s0 = mpc_setup_smem(P.m, P.g, P.p, P.rax, P.nkeep, P.H);
-        cudaFuncSetAttribute(k_mpc_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s0);
+        allow_shared<k_mpc_setup>();
         k_mpc_setup<<<P.m, 128, s0, st>>>(P);
         ++*launches;
     }
     const size_t smem = mpc_smem(P.m, P.g, P.p, P.rax, P.nkeep, P.H, P.warps);
-    cudaFuncSetAttribute(k_mpc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<k_mpc>();
     const int grid = (P.B + P.warps - 1) / P.warps;
     k_mpc<<<grid, 32 * P.warps, smem, st>>>(P);
     ++*launches;

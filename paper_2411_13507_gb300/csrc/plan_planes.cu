@@ -819,7 +819,7 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
         const size_t smem = sizeof(float4) * (size_t)(ob + 1) * (Q.max_orows + EDGE_F4 * Q.max_edges);
         const int fit = (int)(220 * 1024 / (smem + 2 * 1024));
         if (Q.m == 2 && !Q.ub && Q.n_obst >= 24 && fit >= 2) {
-            const cudaError_t ea = cudaFuncSetAttribute(k_planes_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const cudaError_t ea = allow_shared<k_planes_all>();
             if (ea != cudaSuccess) return (int)ea;
             const int nb = (Q.n_obst + ob - 1) / ob, groups = PL_THREADS / ob;
             long long chunks = ((long long)num_sms * (fit < 2 ? fit : 2) + nb - 1) / nb;
