@@ -40,8 +40,8 @@ PDEV float pld32(const void* p, long long i, int f32) {
     return f32 ? ((const float*)p)[i] : (float)((const double*)p)[i];
 }
 
-// Obstacle rows as {A_0, A_1, A_2, b} (FP32, for the inside test), max_orows
-// per obstacle, with row-count checks.
+// Obstacle rows in 3-D as {A_0, A_1, A_2, b} (FP32, for the inside test),
+// max_orows per obstacle, with row-count checks.
 __global__ void k_planes_prep(PlanesParams Q) {
     after_stream<true>();
     const long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -57,9 +57,9 @@ __global__ void k_planes_prep(PlanesParams Q) {
     if (k < nr) {
         const long long r = r0 + k;
         float4 f;
-        f.x = pld32(Q.A, r * Q.m, Q.in_f32);
-        f.y = pld32(Q.A, r * Q.m + 1, Q.in_f32);
-        f.z = Q.m == 3 ? pld32(Q.A, r * Q.m + 2, Q.in_f32) : 0.f;
+        f.x = pld32(Q.A, r * 3, Q.in_f32);
+        f.y = pld32(Q.A, r * 3 + 1, Q.in_f32);
+        f.z = pld32(Q.A, r * 3 + 2, Q.in_f32);
         f.w = pld32(Q.b, r, Q.in_f32);
         reinterpret_cast<float4*>(Q.orow)[u] = f;
     }
@@ -69,20 +69,16 @@ PDEV double pld64(const void* p, long long i, int f32) {
     return f32 ? (double)((const float*)p)[i] : ((const double*)p)[i];
 }
 
-// The interval of t along z0 + t d that every row leaves (t_lo > t_hi: none)
-// and the rows that set its ends (-1 for an infinite end).
-template <int M>
-PDEV void clip_line(const PlanesParams& Q, int r0, int nr, const double* z0, const double* d, double& tlo, double& thi,
-                    int& rlo, int& rhi) {
+// The interval of t along z0 + t d in 3-D that every row leaves (t_lo > t_hi: none).
+PDEV void clip_line(const PlanesParams& Q, int r0, int nr, const double* z0, const double* d, double& tlo, double& thi) {
     const double inf = __longlong_as_double(0x7FF0000000000000ll);
     tlo = -inf;
     thi = inf;
-    rlo = rhi = -1;
     for (int r = 0; r < nr; ++r) {
         double ad = 0.0, az = 0.0;
 #pragma unroll
-        for (int a = 0; a < M; ++a) {
-            const double A = pld64(Q.A, (long long)(r0 + r) * M + a, Q.in_f32);
+        for (int a = 0; a < 3; ++a) {
+            const double A = pld64(Q.A, (long long)(r0 + r) * 3 + a, Q.in_f32);
             ad = fma(A, d[a], ad);
             az = fma(A, z0[a], az);
         }
@@ -94,15 +90,9 @@ PDEV void clip_line(const PlanesParams& Q, int r0, int nr, const double* z0, con
                 thi = -inf;
             }
         } else if (ad > 0.0) {
-            if (slack / ad < thi) {
-                thi = slack / ad;
-                rhi = r;
-            }
+            if (slack / ad < thi) thi = slack / ad;
         } else {
-            if (slack / ad > tlo) {
-                tlo = slack / ad;
-                rlo = r;
-            }
+            if (slack / ad > tlo) tlo = slack / ad;
         }
     }
 }
@@ -126,10 +116,7 @@ PDEV void unit_row(const PlanesParams& Q, int r0, int r, double* n, double& c) {
 
 // One warp per obstacle (3-D): faces (unit normal, offset) and edges,
 // compacted; FP64, rounded to FP32 at the end.  Edge record (4 float4): base point and
-// t_lo; unit direction and t_hi; then in 2-D the unit normals of the rows
-// that end the segment at t_lo and t_hi (zero at an infinite end) and the
-// edge's own unit normal and offset, in 3-D the unit normals of its two
-// facets.
+// t_lo; unit direction and t_hi; the unit normals of its two facets.
 __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
     after_stream<true>();
     constexpr int M = 3;
@@ -165,7 +152,7 @@ __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
             const int c = c0 + lane;
             bool ok = false;
             double z0[3] = {0.0, 0.0, 0.0}, d[3] = {0.0, 0.0, 0.0}, tlo = 0.0, thi = 0.0;
-            int ra = -1, rb = -1, rlo = -1, rhi = -1;  // the edge's own facets, the rows at its ends
+            int ra = -1, rb = -1;  // the edge's own facets
             if (c < ncand) {
                 const int r1 = c / nr, r2 = c - r1 * nr;
                 if (r1 < r2) {
@@ -198,7 +185,7 @@ __global__ void __launch_bounds__(128) k_planes_geom(PlanesParams Q) {
                     }
                 }
                 if (ok) {
-                    clip_line<M>(Q, r0, nr, z0, d, tlo, thi, rlo, rhi);
+                    clip_line(Q, r0, nr, z0, d, tlo, thi);
                     ok = tlo <= thi;
                 }
             }
@@ -235,7 +222,10 @@ PDEV float turn(float ax, float ay, float nx, float ny) {
 // the three unit normals split over them), eight rows at a time.  A chain of
 // FP64 instructions on a pipe that takes about 64 cycles for each of a warp's,
 // so what counts is their number a lane: divisions by 2 rows instead of 7,
-// one root instead of three (500 obstacles: 2.6 + 19 -> 12 us).
+// one root instead of three (500 obstacles: 2.6 + 19 -> 12 us).  Edge record (4
+// float4): base point, turn and t_lo; unit direction, turn and t_hi; the unit
+// normals of the rows that end the segment at t_lo and t_hi (zero at an infinite
+// end); the edge's own unit normal and offset.
 __global__ void __launch_bounds__(128) k_planes_geom2(PlanesParams Q) {
     after_stream<true>();
     const int lane = threadIdx.x & 31, rs = lane & 3;
@@ -463,120 +453,115 @@ PDEV void closest_2d(const float (&v)[NP][2], const Geom<SH>& geo, float (&z)[NP
     }
 }
 
-// The point z of the obstacle nearest to v and its squared distance (0 and v
+// The point z of a 3-D obstacle nearest to v and its squared distance (0 and v
 // itself inside; infinite for an obstacle without a face or an edge).
-template <int M, bool SH>
-PDEV void pair_closest(const float (&v)[M], const Geom<SH>& geo, float (&z)[M], float& d2) {
+PDEV void closest_3d(const float (&v)[3], const Geom<false>& geo, float (&z)[3], float& d2) {
     const float inf = __int_as_float(0x7f800000);
-    if constexpr (M == 2) {
-        const float v1[1][2] = {{v[0], v[1]}};
-        float z1[1][2], d1[1];
-        closest_2d<SH, 1>(v1, geo, z1, d1);
-        z[0] = z1[0][0];
-        z[1] = z1[0][1];
-        d2 = d1[0];
-        return;
-    }
     const int nr = geo.nr;
     bool in = true;
     for (int r = 0; r < nr; ++r) {
         const float4 f = geo.row(r);
-        in = in & (pdot<M>(f, v) - f.w <= 0.f);
+        in = in & (pdot<3>(f, v) - f.w <= 0.f);
     }
     d2 = 0.f;
 #pragma unroll
-    for (int a = 0; a < M; ++a) z[a] = v[a];
-    if (!in) {
-        d2 = inf;
-        if (M == 3) {  // faces whose projection lands inside the obstacle
-            for (int r = 0; r < nr; ++r) {
-                const float4 f = geo.face_of(r);
-                const float sd = pdot<M>(f, v) - f.w;
-                if (!(sd > 0.f) || sd * sd >= d2) continue;
-                float c[M];
+    for (int a = 0; a < 3; ++a) z[a] = v[a];
+    if (in) return;
+    d2 = inf;
+    for (int r = 0; r < nr; ++r) {  // faces whose projection lands inside the obstacle
+        const float4 f = geo.face_of(r);
+        const float sd = pdot<3>(f, v) - f.w;
+        if (!(sd > 0.f) || sd * sd >= d2) continue;
+        float c[3];
 #pragma unroll
-                for (int a = 0; a < M; ++a) c[a] = fmaf(-sd, a == 0 ? f.x : (a == 1 ? f.y : f.z), v[a]);
-                bool ok = true;
-                for (int q = 0; q < nr; ++q) {
-                    if (q == r) continue;
-                    const float4 g = geo.row(q);
-                    const float sv = pdot<M>(g, c) - g.w;
-                    const float mag = fabsf(g.x * c[0]) + fabsf(g.y * c[1]) + fabsf(g.z * c[M - 1]) + fabsf(g.w);
-                    ok = ok && sv <= 8.f * U32P * mag;
-                }
-                if (ok) {
-                    d2 = sd * sd;
-#pragma unroll
-                    for (int a = 0; a < M; ++a) z[a] = c[a];
-                }
-            }
+        for (int a = 0; a < 3; ++a) c[a] = fmaf(-sd, a == 0 ? f.x : (a == 1 ? f.y : f.z), v[a]);
+        bool ok = true;
+        for (int q = 0; q < nr; ++q) {
+            if (q == r) continue;
+            const float4 g = geo.row(q);
+            const float sv = pdot<3>(g, c) - g.w;
+            const float mag = fabsf(g.x * c[0]) + fabsf(g.y * c[1]) + fabsf(g.z * c[2]) + fabsf(g.w);
+            ok = ok && sv <= 8.f * U32P * mag;
         }
-        // edge segments (and their end points, the vertices).  The
-        // candidate is chosen by sign tests, not by comparing nearly
-        // equal distances: a segment whose parameter needs no clamping
-        // holds the projection.  The nearest candidate is the fallback
-        // for what rounding leaves undecided.
-        const int ne = geo.ne;
-        bool found = false;
-        float fb_d2 = inf, fb[M];
+        if (ok) {
+            d2 = sd * sd;
 #pragma unroll
-        for (int a = 0; a < M; ++a) fb[a] = v[a];
-        for (int e = 0; e < ne && !found && !(d2 < inf); ++e) {
-            const float4 e0 = geo.edge_of(e, 0), e1 = geo.edge_of(e, 1);
-            float w[M];
-            w[0] = v[0] - e0.x;
-            w[1] = v[1] - e0.y;
-            if (M == 3) w[M - 1] = v[M - 1] - e0.z;
-            float t = e1.x * w[0];
-            t = fmaf(e1.y, w[1], t);
-            if (M == 3) t = fmaf(e1.z, w[M - 1], t);
-            const float tc = fminf(fmaxf(t, e0.w), e1.w);
-            float c[M], dd = 0.f;
-            c[0] = fmaf(tc, e1.x, e0.x);
-            c[1] = fmaf(tc, e1.y, e0.y);
-            if (M == 3) c[M - 1] = fmaf(tc, e1.z, e0.z);
-#pragma unroll
-            for (int a = 0; a < M; ++a) dd = fmaf(v[a] - c[a], v[a] - c[a], dd);
-            // an unclamped point of an edge whose two facet normals span v - c
-            bool hit = false;
-            if (tc == t) {
-                const float4 e2 = geo.edge_of(e, 2), e3 = geo.edge_of(e, 3);
-                const float wx = v[0] - c[0], wy = v[1] - c[1], wz = v[M - 1] - c[M - 1];
-                // signs of (n_a x w) . d, (w x n_b) . d and (n_a x n_b) . d
-                const float k1 = (e2.y * wz - e2.z * wy) * e1.x + (e2.z * wx - e2.x * wz) * e1.y +
-                                 (e2.x * wy - e2.y * wx) * e1.z;
-                const float k2 = (wy * e3.z - wz * e3.y) * e1.x + (wz * e3.x - wx * e3.z) * e1.y +
-                                 (wx * e3.y - wy * e3.x) * e1.z;
-                float kk = (e2.y * e3.z - e2.z * e3.y) * e1.x + (e2.z * e3.x - e2.x * e3.z) * e1.y +
-                           (e2.x * e3.y - e2.y * e3.x) * e1.z;
-                float s1 = k1, s2 = k2;
-                if (kk < 0.f) {
-                    s1 = -s1;
-                    s2 = -s2;
-                    kk = -kk;
-                }
-                hit = kk > 0.f && s1 >= 0.f && s2 >= 0.f;
-            }
-            if (hit) {
-                found = true;
-                d2 = dd;
-#pragma unroll
-                for (int a = 0; a < M; ++a) z[a] = c[a];
-            } else if (dd < fb_d2) {
-                fb_d2 = dd;
-#pragma unroll
-                for (int a = 0; a < M; ++a) fb[a] = c[a];
-            }
+            for (int a = 0; a < 3; ++a) z[a] = c[a];
         }
-        if (!found && !(d2 < inf)) {
-            d2 = fb_d2;
+    }
+    // edge segments (and their end points, the vertices).  The
+    // candidate is chosen by sign tests, not by comparing nearly
+    // equal distances: a segment whose parameter needs no clamping
+    // holds the projection.  The nearest candidate is the fallback
+    // for what rounding leaves undecided.
+    const int ne = geo.ne;
+    bool found = false;
+    float fb_d2 = inf, fb[3];
 #pragma unroll
-            for (int a = 0; a < M; ++a) z[a] = fb[a];
-        } else if (!found && fb_d2 < d2) {
-            d2 = fb_d2;
+    for (int a = 0; a < 3; ++a) fb[a] = v[a];
+    for (int e = 0; e < ne && !found && !(d2 < inf); ++e) {
+        const float4 e0 = geo.edge_of(e, 0), e1 = geo.edge_of(e, 1);
+        const float w[3] = {v[0] - e0.x, v[1] - e0.y, v[2] - e0.z};
+        float t = e1.x * w[0];
+        t = fmaf(e1.y, w[1], t);
+        t = fmaf(e1.z, w[2], t);
+        const float tc = fminf(fmaxf(t, e0.w), e1.w);
+        float c[3], dd = 0.f;
+        c[0] = fmaf(tc, e1.x, e0.x);
+        c[1] = fmaf(tc, e1.y, e0.y);
+        c[2] = fmaf(tc, e1.z, e0.z);
 #pragma unroll
-            for (int a = 0; a < M; ++a) z[a] = fb[a];
+        for (int a = 0; a < 3; ++a) dd = fmaf(v[a] - c[a], v[a] - c[a], dd);
+        // an unclamped point of an edge whose two facet normals span v - c
+        bool hit = false;
+        if (tc == t) {
+            const float4 e2 = geo.edge_of(e, 2), e3 = geo.edge_of(e, 3);
+            const float wx = v[0] - c[0], wy = v[1] - c[1], wz = v[2] - c[2];
+            // signs of (n_a x w) . d, (w x n_b) . d and (n_a x n_b) . d
+            const float k1 = (e2.y * wz - e2.z * wy) * e1.x + (e2.z * wx - e2.x * wz) * e1.y +
+                             (e2.x * wy - e2.y * wx) * e1.z;
+            const float k2 = (wy * e3.z - wz * e3.y) * e1.x + (wz * e3.x - wx * e3.z) * e1.y +
+                             (wx * e3.y - wy * e3.x) * e1.z;
+            float kk = (e2.y * e3.z - e2.z * e3.y) * e1.x + (e2.z * e3.x - e2.x * e3.z) * e1.y +
+                       (e2.x * e3.y - e2.y * e3.x) * e1.z;
+            float s1 = k1, s2 = k2;
+            if (kk < 0.f) {
+                s1 = -s1;
+                s2 = -s2;
+                kk = -kk;
+            }
+            hit = kk > 0.f && s1 >= 0.f && s2 >= 0.f;
         }
+        if (hit) {
+            found = true;
+            d2 = dd;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) z[a] = c[a];
+        } else if (dd < fb_d2) {
+            fb_d2 = dd;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) fb[a] = c[a];
+        }
+    }
+    if (!found && fb_d2 < d2) {
+        d2 = fb_d2;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) z[a] = fb[a];
+    }
+}
+
+// Either dimension, one point, from global memory.
+template <int M>
+PDEV void pair_closest(const float (&v)[M], const Geom<false>& geo, float (&z)[M], float& d2) {
+    if constexpr (M == 2) {
+        const float v1[1][2] = {{v[0], v[1]}};
+        float z1[1][2], d1[1];
+        closest_2d<false, 1>(v1, geo, z1, d1);
+        z[0] = z1[0][0];
+        z[1] = z1[0][1];
+        d2 = d1[0];
+    } else {
+        closest_3d(v, geo, z, d2);
     }
 }
 
@@ -822,7 +807,7 @@ int launch_planes(const PlanesParams& Q, void* stream, int num_sms, int* launche
             const cudaError_t ea = allow_shared<k_planes_all>();
             if (ea != cudaSuccess) return (int)ea;
             const int nb = (Q.n_obst + ob - 1) / ob, groups = PL_THREADS / ob;
-            long long chunks = ((long long)num_sms * (fit < 2 ? fit : 2) + nb - 1) / nb;
+            long long chunks = (2LL * num_sms + nb - 1) / nb;
             const long long most = (Q.P + groups * PL_NP - 1) / (groups * PL_NP);
             if (chunks > most) chunks = most;
             if (chunks > 65535) chunks = 65535;
