@@ -33,8 +33,9 @@
 //
 // The Hessian and its factor J0 = L^-T depend on the model, dt and the
 // weights only: a small kernel (one CTA per axis block) computes them when
-// those change (the host compares the table with the last call's) and every
-// problem starts from a copy of J0.
+// those change (the host compares the parameters with the last direct call's; a
+// captured call computes its own at every replay) and every problem starts from a
+// copy of J0.
 //
 // One warp per problem: lanes own variable indices (two each up to 64) for
 // the dense steps and strided row ids for the scan; the warp synchronises

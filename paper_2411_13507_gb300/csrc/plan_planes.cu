@@ -672,8 +672,9 @@ __global__ void __launch_bounds__(256) k_planes(PlanesParams Q) {
 // Read per pair from global memory, the 32 obstacles of a warp take 32 lines
 // a load, and those loads bounded the kernel (5000 points x 500 obstacles:
 // 71 us); from shared memory, laid out [entry][obstacle] with one float4 of
-// padding, a load is conflict-free: 53 us, bound by issue (560 instructions a
-// pair, of which 7 edges take 350).  Same arithmetic and results.
+// padding, a load is conflict-free: 53 us, bound by issue (43.8 M warp
+// instructions, 560 a warp of pairs; 70% issue active, 32% of the warps).  Same
+// arithmetic and results.
 constexpr int PL_THREADS = 384, PL_NP = 4;
 
 __global__ void __launch_bounds__(PL_THREADS, 2) k_planes_all(PlanesParams Q, int ob, int chunk) {
