@@ -1425,7 +1425,7 @@ DEVI void record_quads(const float (&x)[M * G], const float* tab, unsigned* dU, 
 }
 
 // Largest |row| over the rows that this state alone fixes (FP32; the other
-// half of such a row is exactly 0).
+// half of such a row is exactly 0), negative for a state that is not finite.
 template <int M, int G, int PD>
 DEVI float single_max(const float (&x)[M * G], const float* tab, bool right) {
     using SS = ScShape<M, G, PD>;
@@ -1436,7 +1436,10 @@ DEVI float single_max(const float (&x)[M * G], const float* tab, bool right) {
 #pragma unroll
         for (int a = 0; a < M; ++a) mx = fmaxf(mx, fabsf(row_half<M, G>(tab + rr * 8 + (right ? 4 : 0), x, a)));
     }
-    return mx;
+    float size = 0.f;
+#pragma unroll
+    for (int e = 0; e < M * G; ++e) size += fabsf(x[e]);
+    return size < __int_as_float(0x7f800000) ? mx : -mx;
 }
 
 // Largest |reach row| of one pair in FP32, by a whole warp (lanes over the rows).
@@ -1667,7 +1670,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
     float* CH = sm;                  // [2T][SC] cost halves, in the place of all of the above once phase 3 is done
     float* magR = sm + sc_front<M, G, PD>(T, DR);  // [2T] band magnitudes
     float* magF = magR + 2 * T;
-    float* smax = magF + 2 * T;      // [2T] largest row fixed by this state alone
+    float* smax = magF + 2 * T;      // [2T] largest row fixed by this state alone, negative: not finite
     float* magC = smax + 2 * T;      // [2T] sum of |cost half| per state-side (cost conditioning):
     float* magC2 = magC + 2 * T;     //      its two parts
     float* xs = magC2 + 2 * T;       // [2T][XS] centred states
@@ -1915,7 +1918,8 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                         if (4 * qd + j < SS::RW) r2[j] = __hmax2(r2[j], __habs2(__hadd2(as_h2(av[j]), as_h2(bv[j]))));
                 }
                 const __half2 rr = __hmax2(__hmax2(r2[0], r2[1]), __hmax2(r2[2], r2[3]));
-                float rm = fmaxf(fmaxf(__low2float(rr), __high2float(rr)) * isc, fmaxf(smax[li], smax[T + lj]));
+                const float si = smax[li], sj = smax[T + lj];
+                float rm = fmaxf(fmaxf(__low2float(rr), __high2float(rr)) * isc, fmaxf(fabsf(si), fabsf(sj)));
                 const float ms = magR[li] + magR[T + lj], b16 = (KR + KHF) * ms + EH * isc, bandR = KR * ms;
                 // what FP16 leaves open, in FP32: a few pairs one after the
                 // other by the whole warp, many (a warp's pass over one pair
@@ -1954,18 +1958,35 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                     }
                     float f2[2] = {NEG_INF, NEG_INF};
                     // rows along an axis: A P_la - b is monotone in P_la, so the
-                    // largest value is that of the extreme coordinate
+                    // largest value is that of the extreme coordinate -- where
+                    // every coordinate is finite.  One that is not makes the other
+                    // axes' rows undefined too (0 times it), as in the loop below.
+                    if ((__float_as_int(si) | __float_as_int(sj)) >= 0) {
 #pragma unroll
-                    for (int a = 0; a < M; ++a) {
-                        float hi = pt[a], lo = pt[a];
+                        for (int a = 0; a < M; ++a) {
+                            float hi = pt[a], lo = pt[a];
 #pragma unroll
-                        for (int l = 1; l < NI; ++l) {
-                            hi = fmaxf(hi, pt[l * M + a]);
-                            lo = fminf(lo, pt[l * M + a]);
+                            for (int l = 1; l < NI; ++l) {
+                                hi = fmaxf(hi, pt[l * M + a]);
+                                lo = fminf(lo, pt[l * M + a]);
+                            }
+                            const float4 bx = box[a];
+                            f2[0] = fmaxf(f2[0], bx.x * hi - bx.y);
+                            f2[1] = fmaxf(f2[1], bx.z * lo - bx.w);
                         }
-                        const float4 bx = box[a];
-                        f2[0] = fmaxf(f2[0], bx.x * hi - bx.y);
-                        f2[1] = fmaxf(f2[1], bx.z * lo - bx.w);
+                    } else {
+#pragma unroll 1
+                        for (int sd = 0; sd < 2 * M; ++sd) {
+                            const float2 ab = reinterpret_cast<const float2*>(box)[sd];
+                            const float ax = sd < 2 ? ab.x : 0.f, ay = sd >> 1 == 1 ? ab.x : 0.f, az = sd > 3 ? ab.x : 0.f;
+#pragma unroll
+                            for (int l = 0; l < NI; ++l) {
+                                float w = ax * pt[l * M];
+                                w = fmaf(ay, pt[l * M + 1], w);
+                                if (M > 2) w = fmaf(az, pt[l * M + 2], w);
+                                f2[l & 1] = fmaxf(f2[l & 1], w - ab.y);
+                            }
+                        }
                     }
                     for (int r = 0; r < s_ng; ++r) {
                         const float4 ab = *reinterpret_cast<const float4*>(Ab + r * 4);
