@@ -1670,7 +1670,10 @@ int plan_wait(plan_ctx* c, plan_info* info) {
     if (d.status == PLAN_ERR_CAPACITY) {
         if (d.detail == DET_SLOTS) c->want_slots = (long long)(d.need_slots + d.need_slots / 4 + 1024);
         if (d.detail == DET_RECHECK) {
+            // blocks stop once the list is full, so the count is only a lower
+            // bound: at least nearly four times the size, for a few retries to do
             long long need = (long long)(d.need_rechecks > d.rechecks ? d.need_rechecks : d.rechecks);
+            if (need < 3 * c->recheckCap) need = 3 * c->recheckCap;
             c->want_rechecks = need + need / 4 + 1024;
         }
         if (d.detail == DET_CUTLIST) {
