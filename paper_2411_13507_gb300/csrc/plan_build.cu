@@ -1425,7 +1425,7 @@ DEVI void record_quads(const float (&x)[M * G], const float* tab, unsigned* dU, 
 }
 
 // Largest |row| over the rows that this state alone fixes (FP32; the other
-// half of such a row is exactly 0), negative for a state that is not finite.
+// half of such a row is exactly 0).
 template <int M, int G, int PD>
 DEVI float single_max(const float (&x)[M * G], const float* tab, bool right) {
     using SS = ScShape<M, G, PD>;
@@ -1436,10 +1436,7 @@ DEVI float single_max(const float (&x)[M * G], const float* tab, bool right) {
 #pragma unroll
         for (int a = 0; a < M; ++a) mx = fmaxf(mx, fabsf(row_half<M, G>(tab + rr * 8 + (right ? 4 : 0), x, a)));
     }
-    float size = 0.f;
-#pragma unroll
-    for (int e = 0; e < M * G; ++e) size += fabsf(x[e]);
-    return size < __int_as_float(0x7f800000) ? mx : -mx;
+    return mx;
 }
 
 // Largest |reach row| of one pair in FP32, by a whole warp (lanes over the rows).
@@ -1468,9 +1465,10 @@ DEVI float lane_reach_f32(const float* xi, const float* xj, const float* tab) {
 }
 
 // Interior control-point halves of one state: point l's coordinate a at
-// dP[l * M + a], zeros up to the next 16-byte quad.
+// dP[l * M + a], zeros up to the next 16-byte quad.  Returns whether the first
+// point is defined: where one of the state's values is NaN, every point is not.
 template <int M, int G, int PD>
-DEVI void point_halves(const float (&x)[M * G], const float* tab, bool right, float* dP) {
+DEVI bool point_halves(const float (&x)[M * G], const float* tab, bool right, float* dP) {
     constexpr int NI = Shape<G, PD>::NI, NP = ScShape<M, G, PD>::NP;
     float v[NP];
 #pragma unroll
@@ -1478,6 +1476,8 @@ DEVI void point_halves(const float (&x)[M * G], const float* tab, bool right, fl
         v[q] = q < NI * M ? row_half<M, G>(tab + (PadTab<G, PD>::ROW_D + q / M) * 8 + (right ? 4 : 0), x, q % M) : 0.f;
 #pragma unroll
     for (int q = 0; q < NP; q += 4) *reinterpret_cast<float4*>(dP + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+    const float sum = M > 2 ? v[0] + v[1] + v[M - 1] : v[0] + v[1];
+    return sum == sum;
 }
 
 template <int M, int G, int PD>
@@ -1670,7 +1670,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
     float* CH = sm;                  // [2T][SC] cost halves, in the place of all of the above once phase 3 is done
     float* magR = sm + sc_front<M, G, PD>(T, DR);  // [2T] band magnitudes
     float* magF = magR + 2 * T;
-    float* smax = magF + 2 * T;      // [2T] largest row fixed by this state alone, negative: not finite
+    float* smax = magF + 2 * T;      // [2T] largest row fixed by this state alone, negative: its points are not defined
     float* magC = smax + 2 * T;      // [2T] sum of |cost half| per state-side (cost conditioning):
     float* magC2 = magC + 2 * T;     //      its two parts
     float* xs = magC2 + 2 * T;       // [2T][XS] centred states
@@ -1840,8 +1840,9 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                 unsigned* dU = (right ? UR : UL) + ls * SU;
                 void* dS = right ? (void*)SCR : (void*)SCL;
                 if (second) {
-                    point_halves<M, G, PD>(x, tab, right, (right ? FR : FL) + ls * SF);
-                    smax[row] = single_max<M, G, PD>(x, tab, right);
+                    const bool defined = point_halves<M, G, PD>(x, tab, right, (right ? FR : FL) + ls * SF);
+                    const float mx = single_max<M, G, PD>(x, tab, right);
+                    smax[row] = defined ? mx : -mx;
                 }
 #pragma unroll
                 for (int e = 0; e < N_; ++e) x[e] *= sc;  // the rows are linear in x, and sc is a power of two
@@ -1959,8 +1960,8 @@ __global__ void __launch_bounds__(256, 3) k_pairs_sc(BuildParams P) {
                     float f2[2] = {NEG_INF, NEG_INF};
                     // rows along an axis: A P_la - b is monotone in P_la, so the
                     // largest value is that of the extreme coordinate -- where
-                    // every coordinate is finite.  One that is not makes the other
-                    // axes' rows undefined too (0 times it), as in the loop below.
+                    // every axis is defined.  One that is not (NaN) makes the other
+                    // axes' rows undefined too, 0 times it, as in the loop below.
                     if ((__float_as_int(si) | __float_as_int(sj)) >= 0) {
 #pragma unroll
                         for (int a = 0; a < M; ++a) {
